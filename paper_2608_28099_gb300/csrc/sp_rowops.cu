@@ -361,149 +361,177 @@ __global__ void swiglu_kernel(PartIn y, int M, int f, int blk, ActOut a) {
     }
 }
 
-// Pooling and the linear head, column-parallel: block (chunk, b) pools 256
-// hidden columns of sequence b (h2 = h1 + y summed over the k rows by four row
-// groups, four columns per thread with 16-byte loads, then mean or last) and
-// writes its partial dot products with every head row to part[b][chunk][C];
-// four classes are reduced at a time (one per row group).
-constexpr int kReadoutCols = 256;
-constexpr int kReadoutGroups = 4;  // row groups of a block (threads = 64 x 4)
+// Pooling and the linear head: block (chunk, b) pools 1024 / RG hidden columns
+// of sequence b (h2 = h1 + y summed over the k rows by RG row groups, four
+// columns per thread with 16-byte loads, then mean or last) and writes its
+// partial dot products with every head row to part[b][chunk][C].  Warp 0 then
+// counts the block; the one that finishes a sequence's last chunk adds the
+// chunks up.
+// Latency-bound: a block is one dependent round trip for its rows, one for the
+// count and one for the sum (3-4 us in all), so the blocks should be few and
+// large: one row group (1024 columns a block, rows four at a time) where that
+// covers the SMs, more groups only where it does not.  With four groups
+// everywhere 96 states of one row took 17.4 us (5 waves of blocks whose threads
+// mostly had no row), 128 of four rows 23.2, 64 of 16 rows 15.1 and 256 of 16
+// rows 48.8 (d = 4096); now 5.8, 8.7, 9.9 and 31.2 us (the last reads 134 MB).
+constexpr int kReadoutThreads = 256;
+constexpr int kReadoutHeads = 4;       // head rows per thread fetched before the wait
+constexpr int kReadoutMinCols = 256;   // columns of a block at RG = 4
 
 __device__ __forceinline__ float4 f4_add(float4 a, float4 b) {
     return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
-__global__ void __launch_bounds__(64 * kReadoutGroups, 2)
-readout_partial_kernel(PartIn y, const float *__restrict__ h1, const float *__restrict__ head_w,
-                       int pool, int k, int d, int C, float *__restrict__ part, size_t sb, size_t sr,
-                       int n_tasks, const float *__restrict__ g_final, float *__restrict__ part_ss,
-                       int *__restrict__ counters, const float *__restrict__ head_b,
-                       float *__restrict__ logits, float eps) {
+template <int RG, int P>
+__global__ void __launch_bounds__(kReadoutThreads, P == 4 ? 2 : 3)
+readout_kernel(PartIn y, const float *__restrict__ h1, const float *__restrict__ head_w, int pool,
+               int k, int d, int C, float *__restrict__ part, size_t sb, size_t sr, int n_tasks,
+               const float *__restrict__ g_final, float *__restrict__ part_ss,
+               int *__restrict__ counters, const float *__restrict__ head_b,
+               float *__restrict__ logits, float eps) {
+    constexpr int CT = kReadoutThreads / RG;   // column threads of a row group
+    constexpr int GW = CT / 32;                // warps of a row group
+    constexpr int H = kReadoutHeads;
     pdl_trigger();
-    __shared__ float4 acc_s[kReadoutGroups][64];
-    __shared__ int is_last;
-    __shared__ float pooled[kReadoutCols];
-    __shared__ float red[4][8];
+    __shared__ float4 acc_s[RG][CT];
+    __shared__ float red[8][H];
+    __shared__ float red_ss[GW];
     const int chunk = blockIdx.x, b = blockIdx.y;
-    const int c = threadIdx.x & 63, rg = threadIdx.x >> 6;
-    const int col = chunk * kReadoutCols + 4 * c;  // d % 4 == 0: a group is all in or all out
+    const int c = threadIdx.x % CT, rg = threadIdx.x / CT;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int col = chunk * 4 * CT + 4 * c;  // d % 4 == 0: a group is all in or all out
     const bool in_d = col < d;
-    const size_t base = (size_t)b * sb;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     head_w += (size_t)(b % n_tasks) * C * d;  // this task's head
     // the head is a constant of the handle, not an output of the previous
     // kernel: the first classes' weights are fetched before the wait
-    const float4 hw0 = (rg < C && in_d) ? *(const float4 *)(head_w + (size_t)rg * d + col)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 hw[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j)
+        hw[j] = (rg + j * RG < C && in_d) ? *(const float4 *)(head_w + (size_t)(rg + j * RG) * d + col) : zero4;
+    const float4 gf = g_final && in_d ? *(const float4 *)(g_final + col) : make_float4(1.f, 1.f, 1.f, 1.f);
     pdl_wait();
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 acc = zero4;
+    // rows rg, rg + RG, ... four at a time (pooling the last row: that row
+    // alone, by group 0), the loads of their h1 values and of up to P partials
+    // issued together
+    const int r_first = pool == SP_POOL_LAST ? k - 1 + rg : rg;
     if (in_d) {
-        // rows rg, rg + G, ... (G row groups) four at a time (all rows when
-        // pooling the last one is a single row), the loads of their h1 values
-        // and of up to four partials each issued together
-        const int r_first = pool == SP_POOL_LAST ? k - 1 : rg;
-        const int r_step = pool == SP_POOL_LAST ? k : kReadoutGroups;
-        if (pool != SP_POOL_LAST || rg == 0) {
-            for (int r0 = r_first; r0 < k; r0 += 4 * r_step) {
-                size_t o[4];
-                bool in[4];
-                float4 v[4];
+        for (int r0 = r_first; r0 < k; r0 += 4 * RG) {
+            size_t o[4];
+            bool in[4];
+            float4 v[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int r = r0 + u * r_step;
-                    in[u] = r < k;
-                    o[u] = base + (size_t)(in[u] ? r : r0) * sr + col;
-                    v[u] = in[u] ? *(const float4 *)(h1 + o[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                for (int i0 = 0; i0 < y.n; i0 += 4) {  // up to four planes per round
-                    float4 pv[4][4];
+            for (int u = 0; u < 4; ++u) {
+                const int r = r0 + u * RG;
+                in[u] = r < k;
+                o[u] = (size_t)b * sb + (size_t)(in[u] ? r : r0) * sr + col;
+                v[u] = in[u] ? *(const float4 *)(h1 + o[u]) : zero4;
+            }
+            for (int i0 = 0; i0 < y.n; i0 += P) {
+                float4 pv[4][P];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                for (int u = 0; u < 4; ++u)
 #pragma unroll
-                        for (int jj = 0; jj < 4; ++jj)
-                            pv[u][jj] = (in[u] && i0 + jj < y.n)
-                                            ? *(const float4 *)(y.y + (size_t)(i0 + jj) * y.stride + o[u])
-                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int jj = 0; jj < P; ++jj)
+                        pv[u][jj] = (in[u] && i0 + jj < y.n)
+                                        ? *(const float4 *)(y.y + (size_t)(i0 + jj) * y.stride + o[u])
+                                        : zero4;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                for (int u = 0; u < 4; ++u)
 #pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) v[u] = f4_add(v[u], pv[u][jj]);
-                }
-                acc = f4_add(acc, f4_add(f4_add(v[0], v[1]), f4_add(v[2], v[3])));
+                    for (int jj = 0; jj < P; ++jj) v[u] = f4_add(v[u], pv[u][jj]);
+            }
+            acc = f4_add(acc, f4_add(f4_add(v[0], v[1]), f4_add(v[2], v[3])));
+        }
+    }
+    if constexpr (RG > 1) {
+        acc_s[rg][c] = acc;
+        __syncthreads();
+        acc = acc_s[0][c];
+#pragma unroll
+        for (int q = 1; q < RG; ++q) acc = f4_add(acc, acc_s[q][c]);
+    }
+    const float dv = pool == SP_POOL_LAST ? 1.f : (float)k;
+    float4 p = make_float4(acc.x / dv, acc.y / dv, acc.z / dv, acc.w / dv);
+    if (g_final) {
+        // LM-head readout: the chunk's share of the pooled row's square sum, and
+        // the pooled values times the final-norm gain (the 1/rms factor is
+        // applied to the finished dot products)
+        if (rg == 0) {
+            const float sq = warp_sum((p.x * p.x + p.y * p.y) + (p.z * p.z + p.w * p.w));
+            if (lane == 0) red_ss[w] = sq;
+        }
+        p = make_float4(p.x * gf.x, p.y * gf.y, p.z * gf.z, p.w * gf.w);
+    }
+    // row group rg takes classes c0 + rg + j RG; its GW warps hold the columns
+    for (int c0 = 0; c0 < C; c0 += H * RG) {
+        if (c0 > 0) {
+            __syncthreads();  // red was read by warp 0
+#pragma unroll
+            for (int j = 0; j < H; ++j) {
+                const int cls = c0 + rg + j * RG;
+                hw[j] = (cls < C && in_d) ? *(const float4 *)(head_w + (size_t)cls * d + col) : zero4;
             }
         }
-    }
-    acc_s[rg][c] = acc;
-    __syncthreads();
-    if (threadIdx.x < 64) {
-        float4 sum = acc_s[0][c];
+        float v[H];
 #pragma unroll
-        for (int q = 1; q < kReadoutGroups; ++q) sum = f4_add(sum, acc_s[q][c]);
-        const float dv = pool == SP_POOL_LAST ? 1.f : (float)k;
-        const float p[4] = {sum.x / dv, sum.y / dv, sum.z / dv, sum.w / dv};
-        if (g_final) {
-            // LM-head readout: the chunk's share of the pooled row's square sum,
-            // and the pooled values times the final-norm gain (the 1/rms factor
-            // is applied to the finished dot products)
-            float sq = in_d ? (p[0] * p[0] + p[1] * p[1]) + (p[2] * p[2] + p[3] * p[3]) : 0.f;
+        for (int j = 0; j < H; ++j)
+            if (c0 + j * RG < C) v[j] = warp_sum((hw[j].x * p.x + hw[j].y * p.y) + (hw[j].z * p.z + hw[j].w * p.w));
+            else v[j] = 0.f;
+        if (lane == 0)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            if ((threadIdx.x & 31) == 0) red[3][4 + (threadIdx.x >> 5)] = sq;
+            for (int j = 0; j < H; ++j) red[w][j] = v[j];
+        __syncthreads();
+        if (w == 0 && lane < H * RG && c0 + lane < C) {
+            const int g = lane % RG, j = lane / RG;
+            float t = 0.f;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) pooled[4 * c + e] = in_d ? p[e] * g_final[col + e] : 0.f;
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) pooled[4 * c + e] = p[e];
+            for (int q = 0; q < GW; ++q) t += red[g * GW + q][j];
+            part[((size_t)b * gridDim.x + chunk) * C + c0 + lane] = t;
         }
     }
-    __syncthreads();
-    if (g_final && threadIdx.x == 0)
-        part_ss[(size_t)b * gridDim.x + chunk] = red[3][4] + red[3][5];
-    // row group rg takes class c0 + rg; its two warps hold the chunk's 256 columns
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int c0 = 0; c0 < C; c0 += kReadoutGroups) {
-        const int cls = c0 + rg;
-        const bool use = cls < C && in_d;
-        const float4 hw = c0 == 0 ? hw0
-                                  : (use ? *(const float4 *)(head_w + (size_t)cls * d + col)
-                                         : make_float4(0.f, 0.f, 0.f, 0.f));
-        float v = use ? (hw.x * pooled[4 * c] + hw.y * pooled[4 * c + 1]) +
-                            (hw.z * pooled[4 * c + 2] + hw.w * pooled[4 * c + 3])
-                      : 0.f;
+    if (w > 0) return;
+    if (g_final && lane == 0) {
+        float t = 0.f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[w >> 1][w & 1] = v;
-        __syncthreads();
-        if (threadIdx.x < kReadoutGroups && c0 + (int)threadIdx.x < C)
-            part[((size_t)b * gridDim.x + chunk) * C + c0 + threadIdx.x] =
-                red[threadIdx.x][0] + red[threadIdx.x][1];
-        __syncthreads();
+        for (int q = 0; q < GW; ++q) t += red_ss[q];
+        part_ss[(size_t)b * gridDim.x + chunk] = t;
     }
-    // the block that finishes sequence b's last chunk adds the chunks' dot
-    // products in chunk order (the bits do not depend on which block is last),
-    // applies the LM-head 1/rms and the bias, and clears the counter
-    __threadfence();  // this block's partials are visible before it is counted
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int before = atomicAdd(counters + b, 1);
-        is_last = before == (int)gridDim.x - 1;
+    // warp 0 wrote the block's partials.  The block that finishes sequence b's
+    // last chunk adds the chunks' dot products in chunk order (the bits do not
+    // depend on which block is last), applies the LM-head 1/rms and the bias,
+    // and clears the counter
+    __syncwarp();
+    int is_last = 0;
+    if (lane == 0) {
+        __threadfence();  // the warp's partials are visible before the block is counted
+        is_last = atomicAdd(counters + b, 1) == (int)gridDim.x - 1;
         if (is_last) counters[b] = 0;
+        __threadfence();  // the other blocks' partials are read after their count
     }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();  // the other blocks' partials are read after their count
+    if (!__shfl_sync(0xffffffffu, is_last, 0)) return;
     const int n_chunks = gridDim.x;
     float inv = 1.f;  // 1 / rms of the pooled row (LM-head readout)
     if (g_final) {
         float ss = 0.f;
+#pragma unroll 8
         for (int j = 0; j < n_chunks; ++j) ss += __ldcg(part_ss + (size_t)b * n_chunks + j);
         inv = rsqrtf(ss / (float)d + eps);
     }
     const float *hb = head_b ? head_b + (size_t)(b % n_tasks) * C : nullptr;
-    for (int cl = threadIdx.x; cl < C; cl += blockDim.x) {
-        float acc = 0.f;
-        for (int j = 0; j < n_chunks; ++j) acc += __ldcg(part + ((size_t)b * n_chunks + j) * C + cl);
-        logits[(size_t)b * C + cl] = acc * inv + (hb ? hb[cl] : 0.f);
+    for (int cl = lane; cl < C; cl += 32) {
+        float t = 0.f;
+#pragma unroll 8
+        for (int j = 0; j < n_chunks; ++j) t += __ldcg(part + ((size_t)b * n_chunks + j) * C + cl);
+        logits[(size_t)b * C + cl] = t * inv + (hb ? hb[cl] : 0.f);
     }
+}
+
+template <int RG, int P, typename... Args>
+cudaError_t launch_readout_t(int B, int d, cudaStream_t st, Args... args) {
+    return launch_k(readout_kernel<RG, P>, dim3(ceil_div(d, 4 * kReadoutThreads / RG), B),
+                    dim3(kReadoutThreads), 0, st, args...);
 }
 
 __global__ void to_act_kernel(const float *__restrict__ x, size_t n, ActOut out) {
@@ -654,21 +682,30 @@ cudaError_t launch_swiglu(PartIn y, int M, int f, int blk, ActOut a, cudaStream_
 
 size_t readout_scratch_bytes(int B, int d, int C) {
     // partial dot products [B][chunks][C], then square sums [B][chunks]
-    return (size_t)B * ceil_div(d, kReadoutCols) * (C + 1) * sizeof(float);
+    return (size_t)B * ceil_div(d, kReadoutMinCols) * (C + 1) * sizeof(float);
 }
 
 cudaError_t launch_readout(PartIn y, const float *h1, const float *head_w, const float *head_b,
                            int pool, int B, int k, int d, int C, float *scratch, float *logits,
                            int *counters, cudaStream_t st, size_t sb, size_t sr, int n_tasks,
                            const float *g_final, float eps) {
-    const int chunks = ceil_div(d, kReadoutCols);
     if (!sb) sb = (size_t)k * d;
     if (!sr) sr = d;
     if (n_tasks < 1) n_tasks = 1;
+    // row groups: none while the grid covers the SMs (see the kernel), else up
+    // to one per row
+    const int rows = pool == SP_POOL_LAST ? 1 : k;
+    int RG = 1;
+    while (RG < 4 && RG < rows && ceil_div(d, 4 * kReadoutThreads / RG) * B < sm_count_cached()) RG *= 2;
+    const int chunks = ceil_div(d, 4 * kReadoutThreads / RG);
     float *ss = g_final ? scratch + (size_t)B * chunks * C : nullptr;
-    return launch_k(readout_partial_kernel, dim3(chunks, B), dim3(64 * kReadoutGroups), 0, st, y, h1,
-                    head_w, pool, k, d, C, scratch, sb, sr, n_tasks, g_final, ss, counters, head_b,
-                    logits, eps);
+#define SP_READOUT_P(RR, PP)                                                                        \
+    launch_readout_t<RR, PP>(B, d, st, y, h1, head_w, pool, k, d, C, scratch, sb, sr, n_tasks, g_final, \
+                             ss, counters, head_b, logits, eps)
+#define SP_READOUT(RR) (y.n <= 1 ? SP_READOUT_P(RR, 1) : y.n == 2 ? SP_READOUT_P(RR, 2) : SP_READOUT_P(RR, 4))
+    return RG == 1 ? SP_READOUT(1) : RG == 2 ? SP_READOUT(2) : SP_READOUT(4);
+#undef SP_READOUT
+#undef SP_READOUT_P
 }
 
 cudaError_t launch_to_act(const float *x, size_t n, ActOut out, cudaStream_t st) {
