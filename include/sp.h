@@ -435,7 +435,9 @@ typedef struct sp_gemm_plan {
     int kblocks_per_cta; /* tile kernel: k-blocks per K split; persistent:
                             units per CTA                                      */
     int splits;          /* fp32 partial planes written                        */
-    int grid;            /* CTAs launched                                      */
+    int grid;            /* persistent: CTAs launched; else (tile, K split) items,
+                            one CTA each (pairs of CTAs take more items than
+                            SMs in turn)                                       */
 } sp_gemm_plan;
 SP_API sp_status sp_debug_gemm_plan(int M, int N, int K, int n_sm, int lo, int schedule,
                                     size_t capacity_bytes, sp_gemm_plan *out);

@@ -1095,7 +1095,7 @@ sp_status sp_project(sp_stream stream, int M, int N, int K, const float *d_x, co
     float *part = (float *)((char *)d_workspace + planes);
     const TcPlan p = tc_plan(M, N, K, sm_count(), workspace_bytes - planes);
     SP_CUDA(launch_to_act(d_x, (size_t)M * K, x.out(true), st));
-    const int bi = bn_index(p.bn);
+    const int bi = bn_index(p.box_rows(true));
     SP_CUDA(launch_gemm_tc(w.map, x.hi[bi], x.lo[bi], p, M, N, K, part, nullptr, st));
     SP_CUDA(launch_sum_partials(PartIn{part, p.splits, (size_t)M * N}, (size_t)M * N, d_y, st));
     return SP_OK;

@@ -35,6 +35,10 @@ struct TcPlan {
     int grid;           // CTAs
     int splits;         // partial planes of Y
     int nt;             // tile kernel: weight tiles per CTA (1, or 2 sharing each activation block)
+    bool pair;          // two CTAs per MMA: the pair kernel runs the tile plan's items
+    int n_sm;
+    // activation rows of one TMA box (the pair kernel's CTAs load half each)
+    int box_rows(bool lo) const { return pair && !lo ? bn / 2 : bn; }
 };
 
 bool encode_kmajor_bf16(CUtensorMap *map, const void *base, int rows, int K, int box_rows);
@@ -173,8 +177,9 @@ struct GemmPlanner {
                   const RopeEpi *rope = nullptr) const {
         cudaError_t e;
         if (use_tc(w, x, path)) {
-            const TcPlan p = tc_plan(M, w.N, w.K, n_sm, y_capacity, lo, sched);
-            const int bi = bn_index(p.bn);
+            TcPlan p = tc_plan(M, w.N, w.K, n_sm, y_capacity, lo, sched);
+            if (inject_stall) p.pair = false;  // the failure-path test is the tile kernel's
+            const int bi = bn_index(p.box_rows(lo));
             e = launch_gemm_tc(w.map, x.hi[bi], x.lo[bi], p, M, w.N, w.K, y, status, st, w.blocked, lo,
                                inject_stall, glu, rope);
             *nsplit = p.splits;

@@ -15,12 +15,14 @@
 // Without the lo plane (template flag LO = false) the activations are plain
 // bf16: half the MMA work and activation traffic, a deeper ring.
 //
-// Two schedules, fp32 partials in planes of Y that the consumers add:
+// Three schedules, fp32 partials in planes of Y that the consumers add:
 //  * tile kernel: one CTA per (tile, K split); split-K when the tiles alone
 //    leave SMs idle.  Roles: warp 0 lane 0 TMA, warp 1 lane 0 MMA, warp 2
 //    TMEM, all eight warps the epilogue (warp w: TMEM lanes 32 (w & 3).., the
 //    column chunks of half w >> 2).  A gate/up projection with one K split can
 //    apply SwiGLU in the epilogue instead of writing partials.
+//  * pair kernel, in the tile kernel's place for the larger tiles: two CTAs per
+//    MMA (cta_group::2), the same (tile, K split) items, persistent.
 //  * persistent stream-K kernel, for tile counts that fill the SMs badly:
 //    one CTA per SM owns the contiguous (tile, k-block) units [c L, (c+1) L)
 //    in tile-major order.  Its weight and activation rings run across tile
@@ -58,8 +60,8 @@ struct TileCfg {
     static constexpr int STAGE = NT * A_BYTES + (LO ? 2 : 1) * B_BYTES;
     static constexpr int STAGES = 196608 / STAGE < 10 ? 196608 / STAGE : 10;  // 192 KB ring
     static constexpr int TMEM_COLS = NT * NB < 32 ? 32 : NT * NB;  // hi and lo halves per tile
-    static constexpr int OFF_POS = STAGES * STAGE + 256;  // rotation epilogue: [BN] (pos, k_new row)
-    static constexpr int SMEM = STAGES * STAGE + 1024 /*align*/ + 256 /*barriers*/ + BN * 8;
+    static constexpr int OFF_POS = STAGES * STAGE + 256;  // rotation epilogue: [BN] positions
+    static constexpr int SMEM = STAGES * STAGE + 1024 /*align*/ + 256 /*barriers*/ + BN * 4;
     static_assert(TMEM_COLS <= 512, "TMEM");
 };
 
@@ -82,6 +84,48 @@ struct TcArgs {
     // rotation epilogue (rope.rope_cs != NULL; RopeEpi)
     RopeEpi rope;
 };
+
+// SwiGLU of four features: silu(gate) * up.
+__device__ __forceinline__ float4 glu4(float4 gt, float4 up) {
+    return make_float4(__fdividef(gt.x, 1.f + __expf(-gt.x)) * up.x, __fdividef(gt.y, 1.f + __expf(-gt.y)) * up.y,
+                       __fdividef(gt.z, 1.f + __expf(-gt.z)) * up.z, __fdividef(gt.w, 1.f + __expf(-gt.w)) * up.w);
+}
+
+// Position of activation row m (0 past the last row); report: record a bad
+// sequence id or length in the status word.
+__device__ __forceinline__ int rope_position(const RopeEpi &p, int m, int M, bool report) {
+    if (m >= M) return 0;
+    const int b = m / p.k, r = m - b * p.k;
+    const SeqRef sq = resolve_seq(p.seq_ids, p.seq_lens, p.lens_by_batch, b, p.n_seqs, p.max_seq_len,
+                                  report ? p.status : nullptr);
+    return sq.len + p.r0 + (p.k_task ? r % p.k_task : r);
+}
+
+// Dims i..i + 3 (x0) and 64 + i.. (x1) of head h of activation row m at position
+// pos: rotated into q or k_new, or copied into v_new.
+__device__ __forceinline__ void rope_store(const RopeEpi &p, int h, int m, int pos, int i, float4 x0, float4 x1) {
+    const int b = m / p.k, kn = b * (p.kn_stride ? p.kn_stride : p.k) + p.r0 + (m - b * p.k);
+    float *dst;
+    if (h < p.Hq + p.Hkv) {
+        const float2 *cs = p.rope_cs + (size_t)pos * 64;
+        const float4 c01 = *(const float4 *)(cs + i), c23 = *(const float4 *)(cs + i + 2);
+        const float c[4] = {c01.x, c01.z, c23.x, c23.z}, sn[4] = {c01.y, c01.w, c23.y, c23.w};
+        const float a0[4] = {x0.x, x0.y, x0.z, x0.w}, a1[4] = {x1.x, x1.y, x1.z, x1.w};
+        float o0[4], o1[4];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+            o0[q4] = a0[q4] * c[q4] - a1[q4] * sn[q4];
+            o1[q4] = a1[q4] * c[q4] + a0[q4] * sn[q4];
+        }
+        x0 = make_float4(o0[0], o0[1], o0[2], o0[3]);
+        x1 = make_float4(o1[0], o1[1], o1[2], o1[3]);
+        dst = h < p.Hq ? p.q + ((size_t)m * p.Hq + h) * 128 : p.k_new + ((size_t)kn * p.Hkv + (h - p.Hq)) * 128;
+    } else {
+        dst = p.v_new + ((size_t)kn * p.Hkv + (h - p.Hq - p.Hkv)) * 128;
+    }
+    *(float4 *)(dst + i) = x0;
+    *(float4 *)(dst + i + 64) = x1;
+}
 
 constexpr int TILE_THREADS = 256;  // warps 0-2 also TMA, MMA and TMEM owner
 
@@ -121,25 +165,13 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
         tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
         tmem_relinquish();
     }
-    // rotation epilogue: the rows' positions and k_new rows, resolved from the
-    // caller's ids and lengths while the main loop runs (they need no wait)
-    int2 *pos_s = (int2 *)(smem + Cfg::OFF_POS);
+    // rotation epilogue: the rows' positions, resolved from the caller's ids and
+    // lengths while the main loop runs (they need no wait)
+    int *pos_s = (int *)(smem + Cfg::OFF_POS);
     const bool rope_on = g.rope.rope_cs != nullptr;
-    if (rope_on && threadIdx.x >= 64) {
-        for (int j = threadIdx.x - 64; j < BN; j += TILE_THREADS - 64) {
-            const int m = m0 + j;
-            int2 pm = make_int2(0, 0);
-            if (m < g.M) {
-                const int b = m / g.rope.k, r = m - b * g.rope.k;
-                const SeqRef sq = resolve_seq(g.rope.seq_ids, g.rope.seq_lens, g.rope.lens_by_batch, b,
-                                              g.rope.n_seqs, g.rope.max_seq_len,
-                                              blockIdx.y == 0 ? g.rope.status : nullptr);
-                pm.x = sq.len + g.rope.r0 + (g.rope.k_task ? r % g.rope.k_task : r);
-                pm.y = b * (g.rope.kn_stride ? g.rope.kn_stride : g.rope.k) + g.rope.r0 + r;
-            }
-            pos_s[j] = pm;
-        }
-    }
+    if (rope_on && threadIdx.x >= 64)
+        for (int j = threadIdx.x - 64; j < BN; j += TILE_THREADS - 64)
+            pos_s[j] = rope_position(g.rope, m0 + j, g.M, blockIdx.y == 0);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -228,8 +260,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
             // lanes i and 64 + i), or copies them for a value head
             float *xb = (float *)smem;
             const int row = quad * 32 + lane, fq = threadIdx.x & 15, cg = threadIdx.x >> 4;
-            const int h = blockIdx.y, i = 4 * fq;  // head = weight tile
-            const int Hq = g.rope.Hq, Hkv = g.rope.Hkv;
+            const int i = 4 * fq;
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 64) {
                 float *buf = xb + ((c0 >> 6) & 1) * (64 * 132);
@@ -246,30 +277,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
                     for (int e = 0; e < 4; ++e) {
                         const int cc = 4 * cg + e, m = m0 + c0 + cc;
                         if (c0 + cc >= BN || m >= g.M) break;
-                        const float4 x0 = ld_shared_v4f(buf + cc * 132 + i);
-                        const float4 x1 = ld_shared_v4f(buf + cc * 132 + 64 + i);
-                        const int2 pm = pos_s[c0 + cc];
-                        float *dst;
-                        if (h < Hq + Hkv) {
-                            const float2 *cs = g.rope.rope_cs + (size_t)pm.x * 64;
-                            const float4 c01 = *(const float4 *)(cs + i), c23 = *(const float4 *)(cs + i + 2);
-                            const float c[4] = {c01.x, c01.z, c23.x, c23.z}, sn[4] = {c01.y, c01.w, c23.y, c23.w};
-                            const float a0[4] = {x0.x, x0.y, x0.z, x0.w}, a1[4] = {x1.x, x1.y, x1.z, x1.w};
-                            float o0[4], o1[4];
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                o0[q4] = a0[q4] * c[q4] - a1[q4] * sn[q4];
-                                o1[q4] = a1[q4] * c[q4] + a0[q4] * sn[q4];
-                            }
-                            dst = h < Hq ? g.rope.q + ((size_t)m * Hq + h) * 128
-                                         : g.rope.k_new + ((size_t)pm.y * Hkv + (h - Hq)) * 128;
-                            *(float4 *)(dst + i) = make_float4(o0[0], o0[1], o0[2], o0[3]);
-                            *(float4 *)(dst + i + 64) = make_float4(o1[0], o1[1], o1[2], o1[3]);
-                        } else {
-                            dst = g.rope.v_new + ((size_t)pm.y * Hkv + (h - Hq - Hkv)) * 128;
-                            *(float4 *)(dst + i) = x0;
-                            *(float4 *)(dst + i + 64) = x1;
-                        }
+                        rope_store(g.rope, blockIdx.y, m, pos_s[c0 + cc], i, ld_shared_v4f(buf + cc * 132 + i),
+                                   ld_shared_v4f(buf + cc * 132 + 64 + i));
                     }
                 }
             }
@@ -302,11 +311,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
                         if (c0 + cc >= BN || m >= g.M) break;
                         const float4 gt = ld_shared_v4f(buf + cc * 132 + 4 * fq);
                         const float4 up = ld_shared_v4f(buf + cc * 132 + 64 + 4 * fq);
-                        act_store4(g.glu, (size_t)m * g.glu_f + feat,
-                                   make_float4(__fdividef(gt.x, 1.f + __expf(-gt.x)) * up.x,
-                                               __fdividef(gt.y, 1.f + __expf(-gt.y)) * up.y,
-                                               __fdividef(gt.z, 1.f + __expf(-gt.z)) * up.z,
-                                               __fdividef(gt.w, 1.f + __expf(-gt.w)) * up.w));
+                        act_store4(g.glu, (size_t)m * g.glu_f + feat, glu4(gt, up));
                     }
                 }
             }
@@ -366,6 +371,281 @@ cudaError_t launch_tile(const CUtensorMap &mw, const CUtensorMap &mh, const CUte
                     g);
 }
 
+
+// ------------------------------------------------------------ pair kernel
+// Large products (128-row tiles with the lo plane, 128- and 256-row tiles
+// without): two CTAs of a cluster on adjacent weight tiles run one
+// tcgen05.mma.cta_group::2 of M = 256.  Each CTA holds its own 128 weight rows
+// and half of the activation rows of the k-block (with the lo plane: rank 0 the
+// hi rows, rank 1 the lo rows), so a stage is 32 KB instead of 48 and an SM
+// writes and reads a third less shared memory per MMA.  Persistent: each pair
+// takes items (row tile, weight tile pair, K split) in turn, with two
+// accumulators in TMEM, so the epilogue of one overlaps the MMAs of the next.
+// Bound by the tensor pipe (the one-CTA tile kernel by shared-memory bandwidth
+// and its exposed epilogue): 4096 rows at d = 4096, Q/K/V hi + lo 325 -> 240 us
+// (1.7 PFLOP/s issued), gate/up 538 -> 440 us (1.88 PFLOP/s), down 303 -> 250 us.
+constexpr int PAIR_THREADS = 384;  // warps 0-7 epilogue, 8 TMA, 9 MMA (rank 0), 10 TMEM
+constexpr int PAIR_TMA = 8, PAIR_MMA = 9, PAIR_TMEM = 10;
+constexpr int EPI_THREADS = 256;
+constexpr int EPI_COLS = 32;                       // columns of an epilogue chunk
+constexpr int EPI_BUF = EPI_COLS * 132 * 4;        // its staging buffer [column][132] fp32
+
+template <int BN, bool LO>
+struct PairCfg {
+    static constexpr int NB = (LO ? 2 : 1) * BN;        // MMA N
+    static constexpr int B_BYTES = NB / 2 * BK * 2;     // this CTA's half of a k-block
+    static constexpr int STAGE = A_BYTES + B_BYTES;
+    static constexpr int STAGES = 196608 / STAGE < 8 ? 196608 / STAGE : 8;
+    static constexpr int TMEM_COLS = 2 * NB;            // two accumulators
+    static constexpr int OFF_EPI = STAGES * STAGE;      // epilogue staging buffer
+    // rotation epilogue: [BN] positions
+    static constexpr int OFF_POS = OFF_EPI + EPI_BUF;
+    static constexpr int OFF_BAR = OFF_POS + BN * 4;
+    static constexpr int SMEM = OFF_BAR + 256 + 1024 /*align*/;
+    // 8 KB of the SM's 228 stay free: the next row kernel's blocks become
+    // resident (and wait) before this kernel ends
+    static_assert(NB <= 256 && TMEM_COLS <= 512 && SMEM <= 219 * 1024, "pair kernel");
+    static_assert((2 * STAGES + 5) * 8 + 8 <= 256, "barriers");
+};
+
+template <int BN, bool LO>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 2)  /* <= 80 registers: see PairCfg::SMEM */
+    gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w,
+                     const __grid_constant__ CUtensorMap map_xhi,
+                     const __grid_constant__ CUtensorMap map_xlo, TcArgs g, int m_tiles, int n_pairs,
+                     int n_items) {
+    using Cfg = PairCfg<BN, LO>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t *full = (uint64_t *)(smem + Cfg::OFF_BAR);  // rank 0's: both CTAs' copies
+    uint64_t *empty = full + Cfg::STAGES;
+    uint64_t *acc_full = empty + Cfg::STAGES;   // [2]
+    uint64_t *acc_empty = acc_full + 2;         // [2], rank 0's: one arrival per CTA
+    uint64_t *fin = acc_empty + 2;
+    uint32_t *tmem_slot = (uint32_t *)(fin + 1);
+    volatile int *abort = (volatile int *)(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int cl = blockIdx.x >> 1, n_cl = gridDim.x >> 1;
+    pdl_trigger();
+
+    if (warp == PAIR_TMA && lane == 0) {
+        for (int s = 0; s < Cfg::STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&acc_full[i], 1);
+            mbar_init(&acc_empty[i], 2);
+        }
+        mbar_init(fin, 1);
+        *abort = 0;
+        fence_mbar_init();
+        prefetch_tmap(&map_w);
+        prefetch_tmap(&map_xhi);
+        prefetch_tmap(&map_xlo);
+    }
+    __syncwarp();
+    // both CTAs' barriers exist before either signals the other's; the TMA warps
+    // go on while TMEM is allocated
+    cluster_arrive();
+    if (warp == PAIR_TMEM) tmem_alloc_pair(tmem_slot, Cfg::TMEM_COLS);
+    cluster_wait();
+    uint32_t tmem = 0;
+    if (warp != PAIR_TMA) {
+        tc_fence_before();
+        asm volatile("bar.sync 2, %0;" ::"n"(PAIR_THREADS - 32) : "memory");
+        tc_fence_after();
+        tmem = *tmem_slot;
+    }
+
+    // item it: row tile it % m_tiles, weight tile pair and K split above it
+    auto item = [&](int it, int &m0, int &tile, int &kb0, int &nkb, int &split) {
+        const int q = it / m_tiles;
+        m0 = (it - q * m_tiles) * BN;
+        split = q / n_pairs;
+        tile = 2 * (q - split * n_pairs) + (int)rank;
+        kb0 = split * g.kb_per_split;
+        nkb = min(g.kb_per_split, g.n_kb - kb0);
+    };
+
+    if (warp == PAIR_TMA && lane == 0) {
+        // each CTA loads its weight rows and its half of the activations; the
+        // bytes of both are counted on rank 0's barrier, which rank 0 arms.
+        // The weights are constant: the first ring of them is requested before
+        // waiting for the previous kernel.
+        const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
+        const CUtensorMap *map_x = LO && rank == 1 ? &map_xlo : &map_xhi;
+        const int x_off = LO ? 0 : (int)rank * (BN / 2);
+        auto load_w = [&](int s, int tile, int kb) {
+            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * Cfg::STAGE);
+            tma_load_2d_pair(smem + s * Cfg::STAGE, &map_w, map_rank(&full[s], 0), g.w_blocked ? 0 : kb * BK,
+                             g.w_blocked ? (tile * g.n_kb + kb) * 128 : tile * 128, pol_w);
+        };
+        int m0, tile, kb0, nkb, split, gi = 0, pre = 0;
+        bool ok = true;
+        if (cl < n_items) {
+            item(cl, m0, tile, kb0, nkb, split);
+            pre = min(nkb, Cfg::STAGES);
+            for (int i = 0; i < pre; ++i) load_w(i, tile, kb0 + i);
+        }
+        pdl_wait();
+        for (int it = cl; ok && it < n_items; it += n_cl) {
+            item(it, m0, tile, kb0, nkb, split);
+            for (int i = 0; i < nkb; ++i, ++gi) {
+                const int s = gi % Cfg::STAGES;
+                if (gi >= pre) {
+                    if (!mbar_wait(&empty[s], ((gi / Cfg::STAGES) & 1) ^ 1, abort, g.wait_ns)) {
+                        ok = false;
+                        break;
+                    }
+                    load_w(s, tile, kb0 + i);
+                }
+                tma_load_2d_pair(smem + s * Cfg::STAGE + A_BYTES, map_x, map_rank(&full[s], 0), (kb0 + i) * BK,
+                                 m0 + x_off, pol_x);
+            }
+        }
+        // nothing may land in this CTA after it is gone: the pair's last loads
+        // are complete when every stage has been read (both CTAs' MMAs), or, after
+        // an abort, once the wait limit has passed
+        for (int j = gi > Cfg::STAGES ? gi - Cfg::STAGES : 0; j < gi; ++j)
+            if (!mbar_wait_drain(&empty[j % Cfg::STAGES], (j / Cfg::STAGES) & 1, g.wait_ns)) break;
+    } else if (warp == PAIR_MMA && lane == 0 && rank == 0) {
+        constexpr uint32_t idesc = idesc_bf16_f32(256, Cfg::NB);
+        int gi = 0, n = 0;
+        bool ok = true;
+        for (int it = cl; ok && it < n_items; it += n_cl, ++n) {
+            int m0, tile, kb0, nkb, split;
+            item(it, m0, tile, kb0, nkb, split);
+            const int buf = n & 1;
+            const uint32_t acc = tmem + (uint32_t)(buf * Cfg::NB);
+            // both CTAs' epilogues have read this accumulator's previous item
+            if (n >= 2 && !mbar_wait_cluster(&acc_empty[buf], ((n >> 1) - 1) & 1, abort, g.wait_ns)) break;
+            tc_fence_after();
+            for (int i = 0; i < nkb; ++i, ++gi) {
+                const int s = gi % Cfg::STAGES;
+                if (!mbar_wait(&full[s], (gi / Cfg::STAGES) & 1, abort, g.wait_ns)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint64_t a = sw128_kmajor_desc(smem + s * Cfg::STAGE);
+                const uint64_t b = sw128_kmajor_desc(smem + s * Cfg::STAGE + A_BYTES);
+#pragma unroll
+                for (int kk = 0; kk < BK / 16; ++kk)  // +32 bytes along K per step (encoded >> 4)
+                    mma_bf16_pair(acc, a + 2 * kk, b + 2 * kk, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                mma_commit_pair(&empty[s]);
+            }
+            if (ok) mma_commit_pair(&acc_full[buf]);
+        }
+        mma_commit_pair(fin);  // every MMA is finished before TMEM and shared memory go away
+        mbar_wait_drain(fin, 0, g.wait_ns);
+    } else if (warp < 8) {
+        // epilogue: warp w reads TMEM lanes 32 (w & 3).. and columns 16 (w >> 2)..
+        // of each 32-column chunk
+        const int quad = warp & 3, half = warp >> 2, row = quad * 32 + lane;
+        const int fq = threadIdx.x & 15, cg = threadIdx.x >> 4;
+        const bool rope_on = g.rope.rope_cs != nullptr;
+        int *pos_s = (int *)(smem + Cfg::OFF_POS);
+        auto epi_all = [](bool ok) {  // all of the epilogue threads' flags
+            int all;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\t"
+                "setp.ne.s32 q, %1, 0;\n\t"
+                "barrier.cta.red.and.pred p, 1, %2, q;\n\t"
+                "selp.s32 %0, 1, 0, p;\n\t}"
+                : "=r"(all)
+                : "r"((int)ok), "n"(EPI_THREADS)
+                : "memory");
+            return all != 0;
+        };
+        auto epi_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory"); };
+        pdl_wait();  // before writing what a previous kernel may still be reading
+        if (rope_on && blockIdx.x == 0)
+            for (int t = threadIdx.x; t < g.rope.n_zero; t += EPI_THREADS) g.rope.zero_ints[t] = 0;
+        int n = 0;
+        for (int it = cl; it < n_items; it += n_cl, ++n) {
+            int m0, tile, kb0, nkb, split;
+            item(it, m0, tile, kb0, nkb, split);
+            const int buf = n & 1;
+            if (rope_on) {
+                // the rows' positions, while the main loop runs
+                for (int j = threadIdx.x; j < BN; j += EPI_THREADS)
+                    pos_s[j] = rope_position(g.rope, m0 + j, g.M, tile == 0);
+            }
+            // one verdict for all epilogue warps (they meet at barriers below)
+            const bool have = epi_all(mbar_wait(&acc_full[buf], (n >> 1) & 1, abort, g.wait_ns));
+            tc_fence_after();
+            const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * Cfg::NB);
+            if (!have) break;
+            if (rope_on || g.glu_f) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < BN; c0 += EPI_COLS) {
+                    // the chunk as [column][132] fp32, then thread (fq, cg) takes rows 4 fq.. and 64 + 4 fq.. of columns
+                    // 2 cg, 2 cg + 1: gate and up of four features, or four rotation pairs
+                    float *xb = (float *)(smem + Cfg::OFF_EPI);
+                    float v[16], u[16] = {};
+                    tmem_ld16(trow + c0 + half * 16, v);
+                    if (LO) tmem_ld16(trow + BN + c0 + half * 16, u);
+                    if (c0 > 0) epi_sync();  // the previous chunk is read
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) xb[(half * 16 + j) * 132 + row] = v[j] + u[j];
+                    epi_sync();
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int cc = 2 * cg + e, m = m0 + c0 + cc;
+                        if (m >= g.M) break;
+                        const float4 x0 = ld_shared_v4f(xb + cc * 132 + 4 * fq);
+                        const float4 x1 = ld_shared_v4f(xb + cc * 132 + 64 + 4 * fq);
+                        if (rope_on)
+                            rope_store(g.rope, tile, m, pos_s[c0 + cc], 4 * fq, x0, x1);
+                        else
+                            act_store4(g.glu, (size_t)m * g.glu_f + (size_t)tile * 64 + 4 * fq, glu4(x0, x1));
+                    }
+                }
+            } else {
+                float *y = g.y + (size_t)split * g.split_stride + (size_t)tile * 128 + row;
+#pragma unroll 1
+                for (int c0 = half * 32; c0 < BN; c0 += 64) {
+                    float v[32], u[32] = {};
+                    tmem_ld32(trow + c0, v);
+                    if (LO) tmem_ld32(trow + BN + c0, u);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const int m = m0 + c0 + j;
+                        if (m < g.M) y[(size_t)m * g.N] = v[j] + u[j];
+                    }
+                }
+            }
+            tc_fence_before();
+            epi_sync();
+            if (threadIdx.x == 0) mbar_arrive_remote(map_rank(&acc_empty[buf], 0));
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort && g.status) atomicOr(g.status, SP_DEV_TIMEOUT);
+    cluster_sync();  // no signal or MMA of the other CTA may still target this one
+    if (warp == PAIR_TMEM) tmem_dealloc_pair(tmem, Cfg::TMEM_COLS);
+}
+
+template <int BN, bool LO>
+cudaError_t launch_pair(const CUtensorMap &mw, const CUtensorMap &mh, const CUtensorMap &ml,
+                        const TcArgs &g, const TcPlan &p, cudaStream_t st) {
+    const int smem = PairCfg<BN, LO>::SMEM;
+    static bool attr_set = false;  // per device process-wide (one device per process here)
+    if (!attr_set) {
+        cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<BN, LO>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    const int n_pairs = p.n_tiles / 2, items = p.m_tiles * n_pairs * p.splits;
+    const int clusters = items < p.n_sm / 2 ? items : p.n_sm / 2;
+    return launch_k(gemm_pair_kernel<BN, LO>, dim3(2 * clusters), dim3(PAIR_THREADS), (size_t)smem, st, mw, mh,
+                    ml, g, p.m_tiles, n_pairs, items);
+}
 
 // ------------------------------------------------------ persistent stream-K
 constexpr int GEMM_THREADS = 224;
@@ -713,6 +993,8 @@ static int planes_for(long long tiles, int n_kb, long long L) {
 TcPlan tc_plan(int M, int N, int K, int n_sm, size_t y_capacity_bytes, bool lo, int sched) {
     TcPlan p;
     p.nt = 1;
+    p.pair = false;
+    p.n_sm = n_sm;
     p.bn = tc_bn_for(M, lo);
     p.m_tiles = ceil_div(M, p.bn);
     p.n_tiles = N / 128;
@@ -764,6 +1046,13 @@ TcPlan tc_plan(int M, int N, int K, int n_sm, size_t y_capacity_bytes, bool lo, 
             return p;
         }
     }
+    // The pair kernel takes 128-row tiles with the lo plane and 256-row tiles
+    // (measured at d = 4096, 1024 rows: Q/K/V 79.9 -> 63.2 us, gate/up 159.4 ->
+    // 124.9 us).  128-row plain tiles are bound by the weights: there the cluster's
+    // start costs as much as the smaller activation half gives until an item has
+    // about 64 k-blocks (4B down at 22: 11.4 -> 11.9 us, 27B down at 91: 32.0 -> 30.8).
+    p.pair = p.n_tiles % 2 == 0 && n_sm >= 2 &&
+             (p.bn == 256 || (p.bn == 128 && (lo || p.kb_per_split >= 64)));
     if (sched == 1) return p;
     if (sched == 2 || (waves > 1 && fill < 0.8)) {
         const long long U = (long long)tiles * p.n_kb;
@@ -775,6 +1064,7 @@ TcPlan tc_plan(int M, int N, int K, int n_sm, size_t y_capacity_bytes, bool lo, 
         const double cost_pk = (double)L + 4.0 + planes * plane_units;
         if ((sched == 2 || cost_pk < cost_tile) && (size_t)planes * M * N * sizeof(float) <= y_capacity_bytes) {
             p.persistent = true;
+            p.pair = false;
             p.units_per_cta = (int)L;
             p.splits = planes;
             p.grid = (int)((U + L - 1) / L);
@@ -837,6 +1127,14 @@ cudaError_t launch_gemm_tc(const CUtensorMap &map_w, const CUtensorMap &map_xhi,
         if (p.persistent || p.splits != 1 || p.bn < 32 || N % 128) return cudaErrorInvalidValue;
         g.glu_f = N / 2;
         g.glu = *glu;
+    }
+    if (p.pair) {
+        switch (p.bn) {
+        case 128: return lo ? launch_pair<128, true>(map_w, map_xhi, map_xlo, g, p, st)
+                            : launch_pair<128, false>(map_w, map_xhi, map_xlo, g, p, st);
+        case 256: return lo ? cudaErrorInvalidValue : launch_pair<256, false>(map_w, map_xhi, map_xlo, g, p, st);
+        default: return cudaErrorInvalidValue;
+        }
     }
     dim3 grid(p.m_tiles, p.n_tiles / p.nt, p.splits);
     if (p.nt == 2) {
