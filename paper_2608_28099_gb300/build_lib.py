@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libsp.so")
 SOURCES = ["sp_api.cu", "sp_rowops.cu", "sp_attn_simt.cu", "sp_gemm_tc.cu", "sp_attend_static.cu",
-           "sp_attn_tc.cu"]
+           "sp_attn_tc.cu", "sp_attn_tok.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xcompiler", "-fvisibility=hidden"]

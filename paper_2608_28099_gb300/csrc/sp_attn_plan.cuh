@@ -1,0 +1,243 @@
+// Shared by the tensor-core attention kernels: the 64-token tile list, its cuts
+// into per-CTA shares, the shared-memory tile layout and the merge of a pair's
+// partials at a kernel's end.
+#pragma once
+
+#include "sp_common.cuh"
+#include "sp_sm100.cuh"
+
+namespace sp {
+
+namespace {
+
+using namespace sm100;
+
+constexpr int DH = 128;
+constexpr int TT = 64;                         // tokens per tile of the list
+constexpr uint32_t GROUP_STRIDE = 2048;        // 8-token groups
+constexpr uint32_t HALF_STRIDE = 1024;         // 64-dim halves within a group
+constexpr int MAX_B = 2048;                    // sequences per launch (tile prefix in smem)
+constexpr int MAX_GRP = 256;                   // groups (cuts table in smem)
+constexpr float RESCALE_LOG2 = 8.f;            // tolerate p <= 2^8 before rescaling O
+constexpr int kStagedSegs = 4;                 // most partials merged through the idle ring
+
+// byte offset of 16-byte chunk c16 (0..15, 8 dims each) of token row `row`
+// (0..63) in a K or V tile
+__device__ __forceinline__ uint32_t kv_off(int row, int c16) {
+    return (uint32_t)((row >> 3) * GROUP_STRIDE + (c16 >> 3) * HALF_STRIDE + (row & 7) * 128 +
+                      (((c16 & 7) ^ (row & 7)) << 4));
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t *>(&v);
+}
+
+__device__ __forceinline__ void named_sync(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// A CTA's piece of one sequence: tiles [t_a, t_a + n) of sequence b, which
+// starts at tile xp of the list and has nt tiles.
+struct Seg {
+    int b, t_a, n, nt, xp;
+};
+
+// Segment holding tile x (x < x_end <= T), clipped at x_end.  prefix[b] is the
+// first tile of sequence b; it grows strictly (every sequence has a tile for
+// its new keys).
+__device__ __forceinline__ Seg seg_at(const int *prefix, int B, int x, int x_end) {
+    int lo = 0, hi = B - 1;
+#pragma unroll 1
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (prefix[mid] <= x) lo = mid;
+        else hi = mid - 1;
+    }
+    Seg s;
+    s.b = lo;
+    s.xp = prefix[lo];
+    s.nt = prefix[lo + 1] - s.xp;
+    s.t_a = x - s.xp;
+    s.n = min(s.nt - s.t_a, x_end - x);
+    return s;
+}
+
+// First tile of group j's share.  A segment boundary inside a share costs the
+// consumers a pipeline drain, the epilogue and the next queries' load, worth
+// about `c` tiles of streaming, so the shares balance tiles + c per sequence:
+// every sequence b gets c virtual tiles in front of its own, the virtual list
+// (T + c B long) is cut evenly, and a cut that lands in a sequence's virtual
+// part moves to that sequence's first tile.  A cut within delta = min(share /
+// 4, SNAP) tiles of a sequence start then moves onto it (a short piece of a
+// sequence would pay a whole boundary).  c falls back to 0 when a share is
+// shorter than c + 1 virtual tiles.  The cuts never decrease; two may meet at a
+// sequence start, and the share between them is then empty (four sequences of 15
+// tiles in eight shares: cuts 0, 0, ...).  Evaluated once per group
+// into a table (cuts[0..n]).
+constexpr int SNAP = 4;
+__device__ __forceinline__ int share_start(const int *prefix, int B, int T, int n, int j, int c) {
+    if (j <= 0) return 0;
+    if (j >= n) return T;
+    if ((long long)T + (long long)c * B < (long long)n * (c + 1)) c = 0;
+    const long long V = (long long)T + (long long)c * B;
+    const long long v = (long long)j * V / n;
+    int lo = 0, hi = B - 1;  // last sequence whose virtual start vpre(b) = prefix[b] + c b is <= v
+#pragma unroll 1
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((long long)prefix[mid] + (long long)c * mid <= v) lo = mid;
+        else hi = mid - 1;
+    }
+    const long long off = v - ((long long)prefix[lo] + (long long)c * lo);
+    int x = off < c ? prefix[lo] : (int)min((long long)prefix[lo] + off - c, (long long)prefix[lo + 1] - 1);
+    const int delta = min(T / n / 4, SNAP);
+    if (delta == 0) return x;
+    lo = 0, hi = B - 1;  // last sequence starting at or before x
+#pragma unroll 1
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (prefix[mid] <= x) lo = mid;
+        else hi = mid - 1;
+    }
+    const int c0 = prefix[lo], c1 = prefix[lo + 1];
+    const int best = (x - c0 <= c1 - x) ? c0 : c1;
+    return abs(best - x) <= delta ? best : x;
+}
+
+// Group whose share holds tile x (0 <= x < T): the largest j with cuts[j] <= x.
+__device__ __forceinline__ int group_of(const int *cuts, int n, int x) {
+    int lo = 0, hi = n - 1;
+#pragma unroll 1
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (cuts[mid] <= x) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// The tile list: prefix[b] = sum_{b' < b} ceil((L_b' + new rows) / TT), and each
+// sequence's cache id and length, resolved once.  By all THREADS threads; wsum
+// holds one int per warp.
+template <int THREADS>
+__device__ __forceinline__ void build_prefix(const AttnArgs &a, int *prefix, int2 *seqs, int *wsum) {
+    const int B = a.B, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = (B + THREADS - 1) / THREADS;
+    const int b0 = min(B, (int)threadIdx.x * per), b1 = min(B, b0 + per);
+    int sum = 0;
+#pragma unroll 1
+    for (int bb = b0; bb < b1; ++bb) {
+        const SeqRef sq = resolve_seq(a.seq_ids, a.seq_lens, a.lens_by_batch, bb, a.kv.n_seqs,
+                                      a.max_seq_len, blockIdx.x == 0 ? a.status : nullptr);
+        seqs[bb] = make_int2(sq.sid, sq.len);
+        const int v = ceil_div(sq.len + a.r0 + a.k, TT);
+        prefix[bb] = v;
+        sum += v;
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int run = incl - sum;
+#pragma unroll 1
+    for (int w = 0; w < warp; ++w) run += wsum[w];
+#pragma unroll 1
+    for (int bb = b0; bb < b1; ++bb) {
+        const int v = prefix[bb];
+        prefix[bb] = run;
+        run += v;
+    }
+    if (threadIdx.x == 0) {
+        int tot = 0;
+#pragma unroll 1
+        for (int w = 0; w < THREADS / 32; ++w) tot += wsum[w];
+        prefix[B] = tot;
+    }
+    __syncthreads();
+}
+
+// Merge of the pair completed by this share's last segment, by the whole
+// CTA: every partial of the pair lands in the idle K/V ring in one
+// round of cp.async copies (O of segment e as [e][row][dh], then (max,
+// sum) as [e][row]), then thread (row, c) combines 16-byte units c, c + 8,
+// c + 16, c + 24 of its row in segment order, in the arithmetic of the
+// register merge above, so the bits do not depend on which path ran.
+// Shared-memory reads are conflict-free and eight lanes store 64
+// contiguous bytes per plane.  Loads through registers would need a
+// dependent round trip per two segments, each waiting behind the other
+// SMs' cache streams.
+// (own: a segment already in place, or -1.  Run by all THREADS threads; good: every wait of the kernel was served; uniform over the CTA.)
+template <int THREADS>
+__device__ __forceinline__ void staged_merge(const AttnArgs &a, uint8_t *stage, int b, int g, int n_seg,
+                                             size_t slot0, bool good, int own = -1) {
+    const int R = a.R, k = a.k, Hkv = a.Hkv;
+    __threadfence();            // the other segments' partials are read after their count
+    float2 *st_ml = (float2 *)(stage + (size_t)n_seg * R * DH * 4);
+    const int units = R * (DH / 4);  // 16-byte units of one segment's O
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < n_seg * units; idx += THREADS) {
+        const int e = idx / units, rem = idx - e * units;
+        if (e != own)
+            cp_async16(stage + (size_t)idx * 16, a.part_o + (slot0 + (size_t)e * Hkv) * R * DH + (size_t)rem * 4);
+    }
+#pragma unroll 1
+    for (int idx = threadIdx.x; idx < n_seg * R; idx += THREADS) {
+        const int e = idx / R, rr = idx - e * R;
+        if (e != own) st_ml[idx] = __ldcg((const float2 *)(a.part_ml + ((slot0 + (size_t)e * Hkv) * R + rr) * 2));
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (good) {
+#pragma unroll 1
+        for (int item = threadIdx.x; item < R * 8; item += THREADS) {
+            const int rr = item >> 3, c = item & 7;
+            float2 ml[kStagedSegs];
+            float4 ov[kStagedSegs][4];
+#pragma unroll
+            for (int e = 0; e < kStagedSegs; ++e) {
+                const int ee = min(e, n_seg - 1);
+                ml[e] = st_ml[ee * R + rr];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    ov[e][q] = ld_shared_v4f(stage + (((size_t)ee * R + rr) * (DH / 4) + c + 8 * q) * 16);
+            }
+            float acc[16], mm = -INFINITY, ll = 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) acc[j] = 0.f;
+#pragma unroll
+            for (int e = 0; e < kStagedSegs; ++e) {
+                if (e >= n_seg) break;
+                const float mn = fmaxf(mm, ml[e].x);
+                if (mn == -INFINITY) continue;
+                const float al = mm == -INFINITY ? 0.f : exp2f(mm - mn);
+                const float wt = ml[e].x == -INFINITY ? 0.f : exp2f(ml[e].x - mn);
+                ll = ll * al + wt * ml[e].y;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    acc[4 * q] = acc[4 * q] * al + wt * ov[e][q].x;
+                    acc[4 * q + 1] = acc[4 * q + 1] * al + wt * ov[e][q].y;
+                    acc[4 * q + 2] = acc[4 * q + 2] * al + wt * ov[e][q].z;
+                    acc[4 * q + 3] = acc[4 * q + 3] * al + wt * ov[e][q].w;
+                }
+                mm = mn;
+            }
+            const float il = ll > 0.f ? 1.f / ll : 0.f;
+            const int hl = rr / k, r = rr - hl * k;
+            const size_t o0 = (((size_t)b * k + r) * a.Hq + g * a.G + hl) * DH;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                act_store4(a.out, o0 + (size_t)(c + 8 * q) * 4,
+                           make_float4(acc[4 * q] * il, acc[4 * q + 1] * il, acc[4 * q + 2] * il,
+                                       acc[4 * q + 3] * il));
+        }
+    }
+}
+
+}  // namespace
+
+}  // namespace sp

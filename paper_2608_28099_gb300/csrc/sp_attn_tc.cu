@@ -64,6 +64,7 @@
 #include <cudaTypedefs.h>
 #include <string.h>
 
+#include "sp_attn_plan.cuh"
 #include "sp_common.cuh"
 #include "sp_sm100.cuh"
 
@@ -73,17 +74,11 @@ namespace {
 
 using namespace sm100;
 
-constexpr int DH = 128;
-constexpr int TT = 64;                         // tokens per tile
 constexpr int STG = 6;                         // K/V ring depth
 constexpr int KV_TILE = TT * DH * 2;           // K or V of one tile, 16 KB
 constexpr int KV_STAGE = 2 * KV_TILE;          // K then V
-constexpr uint32_t GROUP_STRIDE = 2048;        // 8-token groups
-constexpr uint32_t HALF_STRIDE = 1024;         // 64-dim halves within a group
-constexpr int MAX_B = 2048;                    // sequences per launch (tile prefix in smem)
 constexpr int OFF_KV = 0;
 constexpr int OFF_PREFIX = OFF_KV + STG * KV_STAGE;
-constexpr int MAX_GRP = 256;                   // groups (cuts table in smem)
 constexpr int OFF_CUTS = OFF_PREFIX + (MAX_B + 4) * 4;
 constexpr int OFF_BAR = OFF_CUTS + (MAX_GRP + 4) * 4;
 constexpr int OFF_ML = OFF_BAR + 512;           // both warpgroups' (max, sum) per row, 2 KB
@@ -94,8 +89,6 @@ constexpr int OFF_SEQ = OFF_ML + 2048;
 constexpr int SMEM_BYTES = OFF_SEQ + MAX_B * 8 + 1024;
 constexpr int THREADS = 384;                   // 2 softmax warpgroups, 2 producers, 2 MMA
 constexpr int PRODUCER_WARP = 8, MMA_WARP = 9, MMA_WARP1 = 10, PRODUCER_WARP1 = 11;
-constexpr float RESCALE_LOG2 = 8.f;            // tolerate p <= 2^8 before rescaling O
-constexpr int kStagedSegs = 4;                 // most partials merged through the idle ring
 // TMEM columns: S0 [0,64) S1 [64,128) O0 [128,256) O1 [256,384) Qhi [384,448) Qlo [448,512)
 // (Qlo unused with plain queries);
 // P_w (64 bf16 per row) overwrites the first 32 columns of S_w once S_w is read.
@@ -107,22 +100,6 @@ constexpr int BAR_EPI = 1, BAR_SEG = 2;
 
 static_assert(OFF_BAR % 16 == 0 && SMEM_BYTES <= 227 * 1024, "shared memory layout");
 
-// byte offset of 16-byte chunk c16 (0..15, 8 dims each) of token row `row`
-// (0..63) in a K or V tile
-__device__ __forceinline__ uint32_t kv_off(int row, int c16) {
-    return (uint32_t)((row >> 3) * GROUP_STRIDE + (c16 >> 3) * HALF_STRIDE + (row & 7) * 128 +
-                      (((c16 & 7) ^ (row & 7)) << 4));
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t *>(&v);
-}
-
-__device__ __forceinline__ void named_sync(int id, int n) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
 struct Bars {
     uint64_t kv_full[STG], kv_empty[STG], s_full[2], p_full[2], pv_done[2], fin, q_full;  // fin: 2 arrivals
     uint32_t tmem;
@@ -133,81 +110,6 @@ struct Bars {
     int wsum[THREADS / 32];    // tile-prefix scan
 };
 static_assert(sizeof(Bars) <= 512, "barrier block");
-
-// A CTA's piece of one sequence: tiles [t_a, t_a + n) of sequence b, which
-// starts at tile xp of the list and has nt tiles.
-struct Seg {
-    int b, t_a, n, nt, xp;
-};
-
-// Segment holding tile x (x < x_end <= T), clipped at x_end.  prefix[b] is the
-// first tile of sequence b; it grows strictly (every sequence has a tile for
-// its new keys).
-__device__ __forceinline__ Seg seg_at(const int *prefix, int B, int x, int x_end) {
-    int lo = 0, hi = B - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prefix[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    Seg s;
-    s.b = lo;
-    s.xp = prefix[lo];
-    s.nt = prefix[lo + 1] - s.xp;
-    s.t_a = x - s.xp;
-    s.n = min(s.nt - s.t_a, x_end - x);
-    return s;
-}
-
-// First tile of group j's share.  A segment boundary inside a share costs the
-// consumers a pipeline drain, the epilogue and the next queries' load, worth
-// about `c` tiles of streaming, so the shares balance tiles + c per sequence:
-// every sequence b gets c virtual tiles in front of its own, the virtual list
-// (T + c B long) is cut evenly, and a cut that lands in a sequence's virtual
-// part moves to that sequence's first tile.  A cut within delta = min(share /
-// 4, SNAP) tiles of a sequence start then moves onto it (a short piece of a
-// sequence would pay a whole boundary).  c falls back to 0 when a share is
-// shorter than c + 1 virtual tiles, which keeps the cuts strictly increasing
-// (snapping moves them by at most a quarter share).  Evaluated once per group
-// into a table (cuts[0..n]).
-constexpr int SNAP = 4;
-__device__ __forceinline__ int share_start(const int *prefix, int B, int T, int n, int j, int c) {
-    if (j <= 0) return 0;
-    if (j >= n) return T;
-    if ((long long)T + (long long)c * B < (long long)n * (c + 1)) c = 0;
-    const long long V = (long long)T + (long long)c * B;
-    const long long v = (long long)j * V / n;
-    int lo = 0, hi = B - 1;  // last sequence whose virtual start vpre(b) = prefix[b] + c b is <= v
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((long long)prefix[mid] + (long long)c * mid <= v) lo = mid;
-        else hi = mid - 1;
-    }
-    const long long off = v - ((long long)prefix[lo] + (long long)c * lo);
-    int x = off < c ? prefix[lo] : (int)min((long long)prefix[lo] + off - c, (long long)prefix[lo + 1] - 1);
-    const int delta = min(T / n / 4, SNAP);
-    if (delta == 0) return x;
-    lo = 0, hi = B - 1;  // last sequence starting at or before x
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prefix[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    const int c0 = prefix[lo], c1 = prefix[lo + 1];
-    const int best = (x - c0 <= c1 - x) ? c0 : c1;
-    return abs(best - x) <= delta ? best : x;
-}
-
-// Group whose share holds tile x (0 <= x < T): the largest j with cuts[j] <= x.
-__device__ __forceinline__ int group_of(const int *cuts, int n, int x) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (cuts[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
 
 __global__ void __launch_bounds__(THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_k,
@@ -224,44 +126,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int act_warps = (R + 31) / 32;  // softmax warps that own real query rows
     pdl_trigger();
 
-    // ---- the tile list: prefix[b] = sum_{b' < b} ceil((L_b' + k) / TT).
     // Lengths and ids come from the caller, not from the previous kernel, so
     // this runs before pdl_wait.
     int2 *seqs = (int2 *)(smem + OFF_SEQ);  // (sid, len) of sequence b
-    {
-        const int per = (B + THREADS - 1) / THREADS;
-        const int b0 = min(B, (int)threadIdx.x * per), b1 = min(B, b0 + per);
-        int sum = 0;
-        for (int bb = b0; bb < b1; ++bb) {
-            const SeqRef sq = resolve_seq(a.seq_ids, a.seq_lens, a.lens_by_batch, bb, a.kv.n_seqs,
-                                          a.max_seq_len, blockIdx.x == 0 ? a.status : nullptr);
-            seqs[bb] = make_int2(sq.sid, sq.len);
-            const int v = ceil_div(sq.len + a.r0 + k, TT);
-            prefix[bb] = v;
-            sum += v;
-        }
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) bars->wsum[warp] = incl;
-        __syncthreads();
-        int run = incl - sum;
-        for (int w = 0; w < warp; ++w) run += bars->wsum[w];
-        for (int bb = b0; bb < b1; ++bb) {
-            const int v = prefix[bb];
-            prefix[bb] = run;
-            run += v;
-        }
-        if (threadIdx.x == 0) {
-            int tot = 0;
-            for (int w = 0; w < THREADS / 32; ++w) tot += bars->wsum[w];
-            prefix[B] = tot;
-        }
-    }
-    __syncthreads();
+    build_prefix<THREADS>(a, prefix, seqs, bars->wsum);
     const int T = prefix[B];
     const int n_grp = min((int)gridDim.x / Hkv, ceil_div(T, max(1, a.tc_min_tiles)));
     const int grp = blockIdx.x / Hkv, g = blockIdx.x - grp * Hkv;
@@ -859,76 +727,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     if (threadIdx.x == 0 && *abort && a.status) atomicOr(a.status, SP_DEV_TIMEOUT);
     if (bars->fm_merge) {
-        // Merge of the pair completed by this share's last segment, by all 384
-        // threads: every partial of the pair lands in the idle K/V ring in one
-        // round of cp.async copies (O of segment e as [e][row][dh], then (max,
-        // sum) as [e][row]), then thread (row, c) combines 16-byte units c, c + 8,
-        // c + 16, c + 24 of its row in segment order, in the arithmetic of the
-        // register merge above, so the bits do not depend on which path ran.
-        // Shared-memory reads are conflict-free and eight lanes store 64
-        // contiguous bytes per plane.  Loads through registers would need a
-        // dependent round trip per two segments, each waiting behind the other
-        // SMs' cache streams.
-        const int b = bars->fm_b, n_seg = bars->fm_nseg;
-        const size_t slot0 = (size_t)bars->fm_slot0;
-        const bool good = !*abort;  // every wait is over: uniform
-        __threadfence();            // the other segments' partials are read after their count
-        uint8_t *stage = smem + OFF_KV;
-        float2 *st_ml = (float2 *)(stage + (size_t)n_seg * R * DH * 4);
-        const int units = R * (DH / 4);  // 16-byte units of one segment's O
-        for (int idx = threadIdx.x; idx < n_seg * units; idx += THREADS) {
-            const int e = idx / units, rem = idx - e * units;
-            cp_async16(stage + (size_t)idx * 16, a.part_o + (slot0 + (size_t)e * Hkv) * R * DH + (size_t)rem * 4);
-        }
-        for (int idx = threadIdx.x; idx < n_seg * R; idx += THREADS) {
-            const int e = idx / R, rr = idx - e * R;
-            st_ml[idx] = __ldcg((const float2 *)(a.part_ml + ((slot0 + (size_t)e * Hkv) * R + rr) * 2));
-        }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();
-        if (good) {
-            for (int item = threadIdx.x; item < R * 8; item += THREADS) {
-                const int rr = item >> 3, c = item & 7;
-                float2 ml[kStagedSegs];
-                float4 ov[kStagedSegs][4];
-#pragma unroll
-                for (int e = 0; e < kStagedSegs; ++e) {
-                    const int ee = min(e, n_seg - 1);
-                    ml[e] = st_ml[ee * R + rr];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        ov[e][q] = ld_shared_v4f(stage + (((size_t)ee * R + rr) * (DH / 4) + c + 8 * q) * 16);
-                }
-                float acc[16], mm = -INFINITY, ll = 0.f;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) acc[j] = 0.f;
-#pragma unroll
-                for (int e = 0; e < kStagedSegs; ++e) {
-                    if (e >= n_seg) break;
-                    const float mn = fmaxf(mm, ml[e].x);
-                    if (mn == -INFINITY) continue;
-                    const float al = mm == -INFINITY ? 0.f : exp2f(mm - mn);
-                    const float wt = ml[e].x == -INFINITY ? 0.f : exp2f(ml[e].x - mn);
-                    ll = ll * al + wt * ml[e].y;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        acc[4 * q] = acc[4 * q] * al + wt * ov[e][q].x;
-                        acc[4 * q + 1] = acc[4 * q + 1] * al + wt * ov[e][q].y;
-                        acc[4 * q + 2] = acc[4 * q + 2] * al + wt * ov[e][q].z;
-                        acc[4 * q + 3] = acc[4 * q + 3] * al + wt * ov[e][q].w;
-                    }
-                    mm = mn;
-                }
-                const float il = ll > 0.f ? 1.f / ll : 0.f;
-                const int hl = rr / k, r = rr - hl * k;
-                const size_t o0 = (((size_t)b * k + r) * a.Hq + g * a.G + hl) * DH;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    act_store4(a.out, o0 + (size_t)(c + 8 * q) * 4,
-                               make_float4(acc[4 * q] * il, acc[4 * q + 1] * il, acc[4 * q + 2] * il,
-                                           acc[4 * q + 3] * il));
-            }
-        }
+        staged_merge<THREADS>(a, smem + OFF_KV, bars->fm_b, g, bars->fm_nseg, (size_t)bars->fm_slot0, !*abort);
     }
     // the cache stream of the slower CTAs leaves DRAM time for the next
     // projection's weights: this CTA's share goes to L2 (the K/V tiles were
@@ -1010,17 +809,21 @@ bool attention_tc_supported(const AttnArgs &a) {
 
 cudaError_t launch_attention_tc(const AttnArgs &a, const CUtensorMap *map_k,
                                 const CUtensorMap *map_v, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
     CUtensorMap dummy;
     memset(&dummy, 0, sizeof dummy);
-    cudaError_t e = launch_k(attn_tc_kernel, dim3(a.tc_ctas), dim3(THREADS), SMEM_BYTES, st,
-                             map_k ? *map_k : dummy, map_v ? *map_v : dummy, a);
+    cudaError_t e;
+    if (attention_tok_supported(a)) {
+        e = launch_attention_tok(a, map_k ? *map_k : dummy, map_v ? *map_v : dummy, st);
+    } else {
+        static bool attr = false;
+        if (!attr) {
+            e = cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+            if (e != cudaSuccess) return e;
+            attr = true;
+        }
+        e = launch_k(attn_tc_kernel, dim3(a.tc_ctas), dim3(THREADS), SMEM_BYTES, st, map_k ? *map_k : dummy,
+                     map_v ? *map_v : dummy, a);
+    }
     if (e != cudaSuccess || !a.tc_merge_kernel) return e;
     return launch_k(attn_tc_merge_kernel, dim3(a.Hkv, a.B, a.R), dim3(DH), 0, st, a);
 }

@@ -238,12 +238,13 @@ void plan_attention(int B, int Hkv, int k, int max_seq_len, int forced_split, in
 size_t attention_workspace_bytes(int B, int Hkv, int R, int dh, int n_splits, int n_sm);
 // Default fewest tiles per CTA of the tensor-core kernel (64 tokens each).
 constexpr int kAttnMinTiles = 8;
-// Default cost of a segment boundary in the tensor-core kernel, in 64-token
-// tiles (a pipeline drain, the epilogue and the next queries' load).
+// Default cost of a segment boundary in the tensor-core kernels, in 64-token
+// tiles (the epilogue, the first step's row maxima, a merge at a share's end).
+// Tokens-on-M kernel, attention of 4B (contiguous) / 8B paged / 27B long in us:
+// 24.8, 207, 182 at 4; 22.8, 202, 178 at 12; 25.0, 210, 182 at 28.
 constexpr int kAttnSegCost = 12;
-// The same for contiguous caches (cp.async tiles), measured on the 4B shape
-// (B = 16, ~16 tiles per share): 28 gave the attention 40.5 us against 42.6 us
-// at 12; on paged caches 20 was slower than 12 (27B long +1.3 us, 8B paged +6 us).
+// Queries-on-M kernel, contiguous caches (cp.async tiles, 4B shape): 40.5 us at
+// 28 against 42.6 at 12.
 constexpr int kAttnSegCostContiguous = 28;
 // Persistent CTAs of the tensor-core kernel: whole groups of Hkv (one CTA per
 // kv head), as many groups as the SMs hold, at least one.
@@ -256,6 +257,11 @@ cudaError_t launch_attention_simt(const AttnArgs &a, cudaStream_t st);
 bool attention_tc_supported(const AttnArgs &a);
 cudaError_t launch_attention_tc(const AttnArgs &a, const CUtensorMap *map_k,
                                 const CUtensorMap *map_v, cudaStream_t st);
+// The same with tokens on the MMA's M side (sp_attn_tok.cu), where its shared
+// memory plan fits; launched by launch_attention_tc.
+bool attention_tok_supported(const AttnArgs &a);
+cudaError_t launch_attention_tok(const AttnArgs &a, const CUtensorMap &map_k, const CUtensorMap &map_v,
+                                 cudaStream_t st);
 cudaError_t launch_attention_merge(const AttnArgs &a, cudaStream_t st);
 
 // ---------------------------------------------------------------------------

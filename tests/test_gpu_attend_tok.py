@@ -1,0 +1,88 @@
+"""The attention kernel with tokens on the MMA's M side at the edges of its
+work: query rows around the multiples of 16 it pads to, lengths around the
+64-token tiles and 128-token steps, segments of one tile, pairs cut into many
+segments, plain and hi + lo queries, every page size; against the fp64 oracle."""
+import numpy as np
+import pytest
+
+import oracle.sp_oracle as so
+import paper_2608_28099_gb300 as sp
+from paper_2608_28099_gb300 import workloads as wl
+from gpu_util import GpuRun, compare, ensure_built, oracle_logits, rows_tensor
+from test_gpu_parity import _attend
+
+pytestmark = pytest.mark.gpu
+
+LENS = [0, 1, 63, 64, 65, 127, 128, 129, 191, 193, 700, 2100]
+
+
+@pytest.mark.parametrize("hq,hkv,k,page", [
+    (4, 2, 1, 16), (8, 2, 4, 0), (10, 2, 3, 32), (8, 2, 8, 64), (8, 2, 9, 16), (8, 2, 16, 0),
+    (10, 2, 13, 16), (12, 2, 16, 32), (10, 2, 20, 0), (16, 2, 16, 16),
+])
+@pytest.mark.parametrize("split", [0, 64])
+def test_rows_lengths_and_splits(hq, hkv, k, page, split):
+    ensure_built()
+    shape = wl.Shape(256, hq, hkv, 128, 256, k, 2, page_size=page or 16)
+    w = wl.custom(shape, LENS, wl.LAYOUT_PAGED if page else wl.LAYOUT_CONTIGUOUS, 700 + k)
+    rng = np.random.default_rng(k)
+    B = len(LENS)
+    q = (1.5 * rng.standard_normal((B, k, hq, 128))).astype(np.float32)
+    kn, vn = (rng.standard_normal((B, k, hkv, 128)).astype(np.float32) for _ in range(2))
+    q[0, 0, 0] *= 6.0  # rows whose maximum moves (scores of standard deviation 9)
+    q[11, 0, 0] *= 6.0
+    ref = so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn)))
+    out, g = _attend(shape, w, q, kn, vn, 2, split=split)
+    # new values are bf16 (2^-9 of up to 4.5: 9e-3), a new key's score is off by
+    # 1.5 * 2^-9 / sqrt(3) * N(0, 1) (up to 7e-3) and its weight by as much of
+    # itself, times a spread of values of ~1.4: 2e-2 in all, seen 1.2e-2.  A sharp
+    # row's scores are six times that off.
+    err = np.abs(out - ref)
+    sharp = np.zeros(out.shape, bool)
+    sharp[[0, 11], 0, 0] = True
+    assert np.all(err[~sharp] <= 2e-2 * (1 + np.abs(ref[~sharp])))
+    assert np.all(err[sharp] <= 8e-2 * (1 + np.abs(ref[sharp])))
+    if g is not None:
+        for b, L in enumerate(LENS):
+            n = (L + page - 1) // page
+            assert np.array_equal(g[b, :n], w.cache.page_table[b, :n])
+
+
+@pytest.mark.parametrize("hq,k", [(4, 4), (4, 16), (8, 16)])
+def test_empty_share(hq, k):
+    # four sequences of 15 tiles: the first cut between CTA shares snaps to 0, so
+    # the first group of CTAs has nothing to do
+    ensure_built()
+    shape = wl.Shape(256, 2 * hq, 2, 128, 256, k, 2)
+    w = wl.custom(shape, [900 - 4 * (k > 4)] * 4, wl.LAYOUT_PAGED, 710 + k)
+    rng = np.random.default_rng(k)
+    q = rng.standard_normal((4, k, 2 * hq, 128)).astype(np.float32)
+    kn, vn = (rng.standard_normal((4, k, 2, 128)).astype(np.float32) for _ in range(2))
+    ref = so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn)))
+    for _ in range(2):  # the merge counters are clear again after the first call
+        out, _ = _attend(shape, w, q, kn, vn, 2, split=0)
+        np.testing.assert_allclose(out, ref, rtol=1e-2, atol=1e-2)
+
+
+@pytest.mark.parametrize("hq,k,T", [(4, 16, 1), (5, 16, 1), (3, 32, 1), (7, 16, 1), (4, 32, 1), (4, 16, 2)])
+@pytest.mark.parametrize("layout", [wl.LAYOUT_PAGED, wl.LAYOUT_CONTIGUOUS])
+def test_plain_queries_through_classify(hq, k, T, layout):
+    sh = wl.Shape(256, 2 * hq, 2, 128, 512, k, 2)
+    w = wl.custom(sh, [0, 60, 64, 65, 130, 900, 128, 3, 5, 1500], layout, 720 + k, rows_per_seq=True)
+    if T > 1:
+        w = wl.with_tasks(w, T)
+        run = GpuRun(w)
+        torch = run.torch
+        out = torch.empty((len(w.seq_ids), T, 2), dtype=torch.float32, device="cuda")
+        sp.sp_classify(run.model.handle, torch.cuda.current_stream(), len(w.seq_ids), run.ids,
+                       run.cache.seq_lens, run.cache.desc, rows_tensor(torch, w.rows), out)
+        torch.cuda.synchronize()
+        prompts, heads, biases, rows = wl.task_views(w)
+        ref = so.classify_tasks(so.Layer(w.shape, w.weights), w.cache, w.seq_ids, prompts, heads,
+                                biases, rows)
+        for t in range(T):
+            compare(out[:, t].double().cpu().numpy(), ref[:, t], label=f"task {t}")
+    else:
+        run = GpuRun(w)
+        compare(run.logits(), oracle_logits(w), label=f"plain R={hq * k}")
+    run.close()
