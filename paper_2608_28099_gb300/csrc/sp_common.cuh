@@ -316,7 +316,8 @@ cudaError_t launch_readout(PartIn y, const float *h1, const float *head_w, const
 // ---------------------------------------------------------------------------
 // projections
 // ---------------------------------------------------------------------------
-// out = x split into ActOut form (n elements); out = sum of the partials.
+// out = x split into ActOut form (n elements, a multiple of 4, x 16-byte aligned);
+// out = sum of the partials (n a multiple of 4).
 cudaError_t launch_to_act(const float *x, size_t n, ActOut out, cudaStream_t st);
 cudaError_t launch_sum_partials(PartIn y, size_t n, float *out, cudaStream_t st);
 

@@ -534,20 +534,32 @@ cudaError_t launch_readout_t(int B, int d, cudaStream_t st, Args... args) {
                     dim3(kReadoutThreads), 0, st, args...);
 }
 
-__global__ void to_act_kernel(const float *__restrict__ x, size_t n, ActOut out) {
+// n4 vectors of four values.
+__global__ void to_act_kernel(const float4 *__restrict__ x, size_t n4, ActOut out) {
     pdl_trigger();
     pdl_wait();
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4;
          i += (size_t)gridDim.x * blockDim.x)
-        act_store(out, i, x[i]);
+        act_store4(out, 4 * i, x[i]);
 }
 
-__global__ void sum_partials_kernel(PartIn y, size_t n, float *__restrict__ out) {
+// n4 vectors of four values; an output that is not 16-byte aligned is written
+// value by value.
+__global__ void sum_partials_kernel(PartIn y, size_t n4, float *__restrict__ out, int vec) {
     pdl_trigger();
     pdl_wait();
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        out[i] = part_get(y, i);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4;
+         i += (size_t)gridDim.x * blockDim.x) {
+        const float4 v = part_get4(y, 4 * i);
+        if (vec) {
+            *(float4 *)(out + 4 * i) = v;
+        } else {
+            out[4 * i] = v.x;
+            out[4 * i + 1] = v.y;
+            out[4 * i + 2] = v.z;
+            out[4 * i + 3] = v.w;
+        }
+    }
 }
 
 // CUDA-core tiled GEMM: Y[M][N] = X[M][K] W[N][K]^T, fp32 accumulation.
@@ -709,17 +721,20 @@ cudaError_t launch_readout(PartIn y, const float *h1, const float *head_w, const
 }
 
 cudaError_t launch_to_act(const float *x, size_t n, ActOut out, cudaStream_t st) {
-    size_t grid = (n + 255) / 256;
+    if (n % 4 || ((uintptr_t)x & 15)) return cudaErrorInvalidValue;
+    size_t grid = (n / 4 + 255) / 256;
     if (grid > 152 * 16) grid = 152 * 16;
     if (grid == 0) grid = 1;
-    return launch_k(to_act_kernel, dim3((unsigned)grid), dim3(256), 0, st, x, n, out);
+    return launch_k(to_act_kernel, dim3((unsigned)grid), dim3(256), 0, st, (const float4 *)x, n / 4, out);
 }
 
 cudaError_t launch_sum_partials(PartIn y, size_t n, float *out, cudaStream_t st) {
-    size_t grid = (n + 255) / 256;
+    if (n % 4) return cudaErrorInvalidValue;
+    size_t grid = (n / 4 + 255) / 256;
     if (grid > 152 * 16) grid = 152 * 16;
     if (grid == 0) grid = 1;
-    return launch_k(sum_partials_kernel, dim3((unsigned)grid), dim3(256), 0, st, y, n, out);
+    return launch_k(sum_partials_kernel, dim3((unsigned)grid), dim3(256), 0, st, y, n / 4, out,
+                    (int)(((uintptr_t)out & 15) == 0));
 }
 
 cudaError_t launch_gemm_simt(int w_bf16, const void *X, const void *W, float *Y, int M, int N,
