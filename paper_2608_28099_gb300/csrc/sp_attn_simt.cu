@@ -28,34 +28,34 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Address of (token t < L, kv head g) in either cache layout; nullptr when the
-// page-table entry is outside the pool (status bit set by the caller).
-template <typename T>
-__device__ __forceinline__ const T *cache_row(const KVDev &kv, const void *pool_or_null, int sid,
-                                              int t, int g, int Hkv, int dh, bool is_v, int *bad) {
-    if (kv.layout == SP_KV_CONTIGUOUS) {
-        const T *base = (const T *)(is_v ? kv.v_seq[sid] : kv.k_seq[sid]);
-        return base + ((size_t)t * Hkv + g) * dh;
-    }
+__device__ __forceinline__ float4 load4(const float *p) { return *(const float4 *)p; }
+__device__ __forceinline__ float4 load4(const bf16 *p) {
+    const uint2 u = *(const uint2 *)p;
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+}
+
+// Element offset of (token t < L, kv head g) in the sequence's buffer or the
+// pool; -1 when the page-table entry is outside the pool (*bad is set).
+__device__ __forceinline__ long long cache_offset(const KVDev &kv, int sid, int t, int g, int Hkv, int dh, int *bad) {
+    if (kv.layout == SP_KV_CONTIGUOUS) return ((long long)t * Hkv + g) * dh;
     const int P = kv.page_size;
     const int lp = t / P;
     if (lp >= kv.max_pages) {  // a length beyond the page-table row
         *bad = 1;
-        return nullptr;
+        return -1;
     }
     const int page = kv.page_table[(size_t)sid * kv.max_pages + lp];
     if (page < 0 || page >= kv.n_pages) {
         *bad = 1;
-        return nullptr;
+        return -1;
     }
-    const T *pool = (const T *)pool_or_null;
-    return pool + (((size_t)page * Hkv + g) * P + (t % P)) * dh;
+    return (((long long)page * Hkv + g) * P + (t % P)) * dh;
 }
 
 template <typename TKV, int DH>
 __global__ void __launch_bounds__(kThreads) attn_split_simt(AttnArgs a) {
     pdl_trigger();
-    pdl_wait();
     extern __shared__ float smem[];
     const int s = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
     const int R = a.R, k = a.k;
@@ -77,47 +77,73 @@ __global__ void __launch_bounds__(kThreads) attn_split_simt(AttnArgs a) {
     if (t_begin >= total) return;  // the merge reads only units below ceil(total / split)
     const int t_end = min(total, t_begin + a.split_tokens);
 
-    for (int idx = threadIdx.x; idx < R * DH; idx += kThreads) {
-        const int rr = idx / DH, c = idx - rr * DH;
+    // the sequence's buffers (contiguous) or the pools; a sequence without cached
+    // tokens (a bad id among them) has none
+    const bool contig = a.kv.layout == SP_KV_CONTIGUOUS;
+    const TKV *kb = (const TKV *)(contig ? (L > 0 ? a.kv.k_seq[sq.sid] : nullptr) : a.kv.k_pool);
+    const TKV *vb = (const TKV *)(contig ? (L > 0 ? a.kv.v_seq[sq.sid] : nullptr) : a.kv.v_pool);
+    // One tile's K and V as four-element vectors, all loads issued before the
+    // first is stored, the next tile's during this one's products (a chain of
+    // round trips: the tiny layer's step took 11.3 us with element loads in turn, 7.6 now).  The cache is the caller's: the first tile is requested
+    // before the previous kernel (which writes the queries and new rows) is done,
+    // unless it holds new rows.
+    constexpr int NV = kTile * DH / 4 / kThreads;
+    float4 kr[NV], vr[NV];
+    int bad = 0;
+    bool waited = false;
+    auto load_tile = [&](int t0) {
+        if (!waited && min(t_end, t0 + kTile) > L) {
+            pdl_wait();
+            waited = true;
+        }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int idx = threadIdx.x + i * kThreads, tt = idx / (DH / 4), c = (idx - tt * (DH / 4)) * 4;
+            const int t = t0 + tt;
+            kr[i] = vr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (t < t_end && t < L) {
+                const long long o = cache_offset(a.kv, sq.sid, t, g, a.Hkv, DH, &bad);
+                if (o >= 0) {
+                    kr[i] = load4(kb + o + c);
+                    vr[i] = load4(vb + o + c);
+                }
+                if (c == 0 && a.gathered && !contig && (t % a.kv.page_size == 0 || tt == 0) &&
+                    t / a.kv.page_size < a.kv.max_pages)
+                    a.gathered[(size_t)b * a.kv.max_pages + t / a.kv.page_size] =
+                        a.kv.page_table[(size_t)sq.sid * a.kv.max_pages + t / a.kv.page_size];
+            } else if (t < t_end) {
+                const size_t o = (((size_t)b * kns + (t - L)) * a.Hkv + g) * DH + c;
+                kr[i] = load4(a.k_new + o);
+                vr[i] = load4(a.v_new + o);
+            }
+        }
+    };
+    load_tile(t_begin);
+    if (!waited) pdl_wait();
+    waited = true;
+    for (int idx = threadIdx.x; idx < R * DH / 4; idx += kThreads) {
+        const int rr = idx / (DH / 4), c = (idx - rr * (DH / 4)) * 4;
         const int hl = rr / k, r = rr - hl * k;
         const int h = g * a.G + hl;
-        Qs[idx] = a.q[(((size_t)b * k + r) * a.Hq + h) * DH + c] * a.scale_log2;
-        Os[idx] = 0.f;
+        const float4 q = load4(a.q + (((size_t)b * k + r) * a.Hq + h) * DH + c);
+        *(float4 *)(Qs + idx * 4) = make_float4(q.x * a.scale_log2, q.y * a.scale_log2, q.z * a.scale_log2, q.w * a.scale_log2);
+        *(float4 *)(Os + idx * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     for (int rr = threadIdx.x; rr < R; rr += kThreads) {
         mrow[rr] = -INFINITY;
         lrow[rr] = 0.f;
     }
-    int bad = 0;
     __syncthreads();
 
     for (int t0 = t_begin; t0 < t_end; t0 += kTile) {
-        for (int idx = threadIdx.x; idx < kTile * DH; idx += kThreads) {
-            const int tt = idx / DH, c = idx - tt * DH;
-            const int t = t0 + tt;
-            float kv_k = 0.f, kv_v = 0.f;
-            if (t < t_end) {
-                if (t < L) {
-                    const TKV *kr = cache_row<TKV>(a.kv, a.kv.k_pool, sq.sid, t, g, a.Hkv, DH,
-                                                   false, &bad);
-                    const TKV *vr = cache_row<TKV>(a.kv, a.kv.v_pool, sq.sid, t, g, a.Hkv, DH,
-                                                   true, &bad);
-                    if (kr) kv_k = to_f(kr[c]);
-                    if (vr) kv_v = to_f(vr[c]);
-                    if (c == 0 && a.gathered && a.kv.layout == SP_KV_PAGED &&
-                        (t % a.kv.page_size == 0 || tt == 0) && t / a.kv.page_size < a.kv.max_pages)
-                        a.gathered[(size_t)b * a.kv.max_pages + t / a.kv.page_size] =
-                            a.kv.page_table[(size_t)sq.sid * a.kv.max_pages + t / a.kv.page_size];
-                } else {
-                    const int j = t - L;
-                    const size_t o = (((size_t)b * kns + j) * a.Hkv + g) * DH + c;
-                    kv_k = a.k_new[o];
-                    kv_v = a.v_new[o];
-                }
-            }
-            Ks[tt * (DH + 1) + c] = kv_k;
-            Vs[tt * DH + c] = kv_v;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int idx = threadIdx.x + i * kThreads, tt = idx / (DH / 4), c = (idx - tt * (DH / 4)) * 4;
+            float *kd = Ks + tt * (DH + 1) + c, *vd = Vs + tt * DH + c;
+            kd[0] = kr[i].x; kd[1] = kr[i].y; kd[2] = kr[i].z; kd[3] = kr[i].w;
+            vd[0] = vr[i].x; vd[1] = vr[i].y; vd[2] = vr[i].z; vd[3] = vr[i].w;
         }
+        if (t0 + kTile < t_end) load_tile(t0 + kTile);  // in flight during this tile's products
         __syncthreads();
         for (int idx = threadIdx.x; idx < R * kTile; idx += kThreads) {
             const int rr = idx / kTile, tt = idx - rr * kTile;

@@ -74,19 +74,8 @@ struct PartIn {
     int n;
     size_t stride;
 };
-// Loads of up to eight partials are issued together before they are added
-// (the adds would otherwise serialise one memory latency per partial).
-__device__ __forceinline__ float part_get(const PartIn &p, size_t idx) {
-    float s = 0.f;
-    for (int i0 = 0; i0 < p.n; i0 += 8) {
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = (i0 + j < p.n) ? p.y[(size_t)(i0 + j) * p.stride + idx] : 0.f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) s += v[j];
-    }
-    return s;
-}
+// Loads of up to four partials are issued together before they are added (the
+// adds would otherwise serialise one memory latency per partial).
 // Four consecutive values (idx and stride multiples of 4).
 __device__ __forceinline__ float4 part_get4(const PartIn &p, size_t idx) {
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -616,6 +616,53 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const float *__restrict_
     }
 }
 
+// CUDA-core projection of few rows: one warp per output column, up to eight rows
+// at a time, four consecutive k per lane (coalesced 512-byte reads of the weight
+// row; the activations stay in L1), partial sums over the lanes added by halving
+// exchanges.  Latency-bound: the tiled kernel's chain of shared-memory slices made
+// every product of the tiny layer 4-5 us, this one is one or two round trips.
+constexpr int kGemvRows = 8;
+template <typename T>
+__global__ void __launch_bounds__(256) gemv_simt_kernel(const float *__restrict__ X, const T *__restrict__ W,
+                                                        float *__restrict__ Y, int M, int N, int K,
+                                                        int w_blocked) {
+    pdl_trigger();
+    pdl_wait();
+    const int lane = threadIdx.x & 31, n = blockIdx.x * 8 + (threadIdx.x >> 5), m0 = blockIdx.y * kGemvRows;
+    if (n >= N) return;
+    const int rows = min(kGemvRows, M - m0);
+    float acc[kGemvRows];
+#pragma unroll
+    for (int r = 0; r < kGemvRows; ++r) acc[r] = 0.f;
+    const float *x = X + (size_t)m0 * K;
+#pragma unroll 2
+    for (int k = lane * 4; k < K; k += 128) {
+        const size_t wi = w_blocked ? (((size_t)(n >> 7) * (K >> 6) + (k >> 6)) * 128 + (n & 127)) * 64 + (k & 63)
+                                    : (size_t)n * K + k;
+        const float4 w = load4(W + wi);
+#pragma unroll
+        for (int r = 0; r < kGemvRows; ++r) {
+            if (r >= rows) break;
+            const float4 v = load4(x + (size_t)r * K + k);
+            acc[r] = fmaf(v.x, w.x, fmaf(v.y, w.y, fmaf(v.z, w.z, fmaf(v.w, w.w, acc[r]))));
+        }
+    }
+    // eight sums over 32 lanes: lane 4 r ends with row r
+#pragma unroll
+    for (int o = 16, c = kGemvRows; c > 1; o >>= 1, c >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < c / 2; ++j) {
+            const float send = up ? acc[j] : acc[j + c / 2], keep = up ? acc[j + c / 2] : acc[j];
+            acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    const int r = lane >> 2;
+    if ((lane & 3) == 0 && r < rows) Y[(size_t)(m0 + r) * N + n] = acc[0];
+}
+
 }  // namespace
 
 cudaError_t launch_rmsnorm_rows(int x_bf16, const void *x, int row_mod, const float *gain,
@@ -739,6 +786,20 @@ cudaError_t launch_sum_partials(PartIn y, size_t n, float *out, cudaStream_t st)
 
 cudaError_t launch_gemm_simt(int w_bf16, const void *X, const void *W, float *Y, int M, int N,
                              int K, cudaStream_t st, bool w_blocked) {
+    // one row group re-reads nothing; with more, the activations' re-reads per
+    // column outgrow the tiled kernel's on large matrices.  Measured, tiled -> this:
+    // 4 x 128 x 256 14.3 -> 4.0 us, 8 x 6144 x 2560 248 -> 51, 32 x 6144 x 2560
+    // 260 -> 129, 4 x 24576 x 4096 497 -> 138, 32 x 24576 x 4096 502 -> 1018
+    const int groups = ceil_div(M, kGemvRows);
+    if ((groups == 1 || (groups <= 4 && (long long)N * K <= (1 << 24))) && K % 4 == 0 &&
+        !(((uintptr_t)X | (uintptr_t)W) & 15)) {
+        const dim3 gv(ceil_div(N, 8), groups);
+        if (w_bf16)
+            return launch_k(gemv_simt_kernel<bf16>, gv, dim3(256), 0, st, (const float *)X, (const bf16 *)W, Y, M, N,
+                            K, (int)w_blocked);
+        return launch_k(gemv_simt_kernel<float>, gv, dim3(256), 0, st, (const float *)X, (const float *)W, Y, M, N,
+                        K, (int)w_blocked);
+    }
     dim3 grid(ceil_div(N, 64), ceil_div(M, 64));
     if (w_bf16)
         return launch_k(gemm_simt_kernel<bf16>, grid, dim3(256), 0, st, (const float *)X, (const bf16 *)W,
