@@ -622,6 +622,9 @@ static sp_status recursive_impl(sp_handle *h, cudaStream_t st, int batch, const 
     const bool tc_down = h->gemm.use_tc(h->w_down, h->a, h->opt_gemm);
     for (bool &u : h->ev_used) u = false;
     int ns = 1;
+    // SwiGLU in the gate/up projection's epilogue where it runs unsplit
+    const ActOut a_out = h->a.out(tc_down);
+    const bool glu = h->gu_blk == 64 && h->gemm.glu_fusable(h->w_gu, h->n, h->opt_gemm, B, true);
     SP_CUDA(launch_rmsnorm_rows(wb, d_hidden, 0, h->g_h, c.rms_eps, B, d, h->xh.out(tc_fc), st));
     ++launches;
     // one split plan for every step: keys extend to L_b + k at the last step
@@ -673,10 +676,13 @@ static sp_status recursive_impl(sp_handle *h, cudaStream_t st, int batch, const 
         SP_CUDA(launch_residual_norm(0, PartIn{h->y, ns, Bd}, h->xrows, 0, h->g_post, c.rms_eps, B, d,
                                      h->h1, h->n.out(tc_gu), st));
         ++launches;
-        s = h->gemm.run(wb, h->opt_gemm, h->n, h->w_gu, h->y, B, h->status, st, &launches, &ns);
+        s = h->gemm.run(wb, h->opt_gemm, h->n, h->w_gu, h->y, B, h->status, st, &launches, &ns, true, 0,
+                        glu ? &a_out : nullptr);
         if (s != SP_OK) return fail(s, "gate/up projection launch failed");
-        SP_CUDA(launch_swiglu(PartIn{h->y, ns, (size_t)B * 2 * f}, B, f, h->gu_blk, h->a.out(tc_down), st));
-        ++launches;
+        if (!glu) {
+            SP_CUDA(launch_swiglu(PartIn{h->y, ns, (size_t)B * 2 * f}, B, f, h->gu_blk, a_out, st));
+            ++launches;
+        }
         s = h->gemm.run(wb, h->opt_gemm, h->a, h->w_down, h->y, B, h->status, st, &launches, &ns);
         if (s != SP_OK) return fail(s, "down projection launch failed");
         // a_i = h1 + W_down a -> h2_all[i]; RMSNorm(a_i; g_h) is the next step's fusion input

@@ -159,7 +159,7 @@ struct GemmPlanner {
     bool glu_fusable(const WeightMat &w, const ActBuf &x, int path, int M, bool lo) const {
         if (!use_tc(w, x, path)) return false;
         const TcPlan p = tc_plan(M, w.N, w.K, n_sm, y_capacity, lo, sched);
-        return !p.persistent && p.splits == 1 && p.bn >= 32;
+        return !p.persistent && p.splits == 1;
     }
     // Would the Q/K/V projection run with the rotation epilogue (one CTA per
     // weight tile = head, no K split)?

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
             }
         }
     } else if (g.glu_f) {
-        if constexpr (BN >= 32) {
+        {
             // SwiGLU epilogue, per 64-column chunk: every warp puts 32 columns of
             // its 32 rows (TMEM lanes) into the idle ring as [column][132] fp32
             // (two buffers), then thread (fq, cg) forms features 4 fq..4 fq + 3
@@ -296,7 +296,15 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 64) {
                 float *buf = xb + ((tj * ((BN + 63) / 64) + (c0 >> 6)) & 1) * (64 * 132);  // chunks alternate
-                if (have && c0 + half * 32 < BN) {
+                if constexpr (BN == 16) {
+                    if (have && half == 0) {
+                        float v[16], u[16] = {};
+                        tmem_ld16(trow, v);
+                        if (LO) tmem_ld16(trow + BN, u);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) buf[j * 132 + row] = v[j] + u[j];
+                    }
+                } else if (have && c0 + half * 32 < BN) {
                     float v[32], u[32] = {};
                     tmem_ld32(trow + c0 + half * 32, v);
                     if (LO) tmem_ld32(trow + BN + c0 + half * 32, u);
@@ -305,9 +313,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
                 }
                 __syncthreads();
                 if (have) {
+                    constexpr int E = BN < 64 ? BN / 16 : 4;  // columns per thread of a chunk
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int cc = 4 * cg + e, m = m0 + c0 + cc;
+                    for (int e = 0; e < E; ++e) {
+                        const int cc = E * cg + e, m = m0 + c0 + cc;
                         if (c0 + cc >= BN || m >= g.M) break;
                         const float4 gt = ld_shared_v4f(buf + cc * 132 + 4 * fq);
                         const float4 up = ld_shared_v4f(buf + cc * 132 + 64 + 4 * fq);
@@ -1124,7 +1133,7 @@ cudaError_t launch_gemm_tc(const CUtensorMap &map_w, const CUtensorMap &map_xhi,
         g.rope = *rope;
     }
     if (glu) {
-        if (p.persistent || p.splits != 1 || p.bn < 32 || N % 128) return cudaErrorInvalidValue;
+        if (p.persistent || p.splits != 1 || N % 128) return cudaErrorInvalidValue;
         g.glu_f = N / 2;
         g.glu = *glu;
     }
