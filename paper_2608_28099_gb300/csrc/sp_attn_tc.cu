@@ -364,77 +364,80 @@ __global__ void __launch_bounds__(THREADS, 1)
         // PV_i (after softmax i) and S_{i+2} (reusing S buffer w).  PV_i does not
         // wait for any later tile's data, so stage i is released as soon as its
         // softmax is done.
+        // (by the whole warp, the instructions under `lead`: see elect_one)
         const int w = warp - MMA_WARP;
-        if (lane == 0) {
-            constexpr uint32_t idesc_s = idesc_bf16_f32(128, TT);
-            constexpr uint32_t idesc_o = idesc_bf16_f32_bmn(128, DH);
-            const uint32_t s_tmem = tmem + (uint32_t)(w * TT);  // S_w; P_w over its first half
-            const uint32_t o_tmem = tmem + O_COL + (uint32_t)(w * DH);
-            auto issue_s = [&](int cst) {
-                const uint8_t *K = smem + OFF_KV + cst * KV_STAGE;
+        const bool lead = elect_one();
+        constexpr uint32_t idesc_s = idesc_bf16_f32(128, TT);
+        constexpr uint32_t idesc_o = idesc_bf16_f32_bmn(128, DH);
+        const uint32_t s_tmem = tmem + (uint32_t)(w * TT);  // S_w; P_w over its first half
+        const uint32_t o_tmem = tmem + O_COL + (uint32_t)(w * DH);
+        const uint64_t dk0 = sw128_kmajor_desc_sbo(smem + OFF_KV, GROUP_STRIDE);
+        const uint64_t dv0 = sw128_mnmajor_desc2(smem + OFF_KV + KV_TILE, HALF_STRIDE, GROUP_STRIDE);
+        auto issue_s = [&](int cst) {
+            const uint64_t dk = dk0 + (uint32_t)(cst * (KV_STAGE >> 4));
+            if (!lead) return;
 #pragma unroll
-                for (int kk = 0; kk < DH / 16; ++kk) {
-                    // 16 dims = 32 B along a 128-byte row of dim half kk / 4
-                    const uint64_t bk =
-                        sw128_kmajor_desc_sbo(K + (kk >> 2) * HALF_STRIDE, GROUP_STRIDE) +
-                        (uint64_t)((kk & 3) * 2);
-                    // 16 dims of Q = 8 TMEM columns
-                    mma_bf16_ts(s_tmem, tmem + QHI_COL + (uint32_t)(kk * 8), bk, idesc_s,
-                                kk > 0 ? 1u : 0u);
-                    if (!a.tc_q_plain)
-                        mma_bf16_ts(s_tmem, tmem + QLO_COL + (uint32_t)(kk * 8), bk, idesc_s, 1u);
-                }
-                mma_commit(&bars->s_full[w]);
-            };
-            bool ok = true;
-            int ci0 = 0, kw = 0, j = 0;
-            for (int x = x0; ok && x < x1; ++j) {
-                const Seg sg = seg_at(prefix, B, x, x1);
-                x += sg.n;
-                if (!mbar_wait(&bars->q_full, (uint32_t)(j & 1), abort)) break;
-                tc_fence_after();
-                if (w < sg.n) {
-                    const int cw = ci0 + w;
-                    ok = mbar_wait(&bars->kv_full[cw % STG], (cw / STG) & 1, abort);
-                    if (ok) {
-                        tc_fence_after();
-                        fence_proxy_async();  // cp.async data -> tensor-core reads
-                        issue_s(cw % STG);
-                    }
-                }
-                for (int i = w; ok && i < sg.n; i += 2, ++kw) {
-                    if (!mbar_wait(&bars->p_full[w], (uint32_t)(kw & 1), abort)) {
-                        ok = false;
-                        break;
-                    }
+            for (int kk = 0; kk < DH / 16; ++kk) {
+                // 16 dims = 32 B along a 128-byte row of dim half kk / 4
+                const uint64_t bk = dk + (uint64_t)((kk >> 2) * (HALF_STRIDE >> 4) + (kk & 3) * 2);
+                // 16 dims of Q = 8 TMEM columns
+                mma_bf16_ts(s_tmem, tmem + QHI_COL + (uint32_t)(kk * 8), bk, idesc_s,
+                            kk > 0 ? 1u : 0u);
+                if (!a.tc_q_plain)
+                    mma_bf16_ts(s_tmem, tmem + QLO_COL + (uint32_t)(kk * 8), bk, idesc_s, 1u);
+            }
+            mma_commit(&bars->s_full[w]);
+        };
+        bool ok = true;
+        int ci0 = 0, kw = 0, j = 0;
+        for (int x = x0; ok && x < x1; ++j) {
+            const Seg sg = seg_at(prefix, B, x, x1);
+            x += sg.n;
+            if (!mbar_wait_warp(&bars->q_full, (uint32_t)(j & 1), abort)) break;
+            tc_fence_after();
+            if (w < sg.n) {
+                const int cw = ci0 + w;
+                ok = mbar_wait_warp(&bars->kv_full[cw % STG], (cw / STG) & 1, abort);
+                if (ok) {
                     tc_fence_after();
-                    const int cst = (ci0 + i) % STG;
-                    const uint8_t *V = smem + OFF_KV + cst * KV_STAGE + KV_TILE;
+                    fence_proxy_async();  // cp.async data -> tensor-core reads
+                    issue_s(cw % STG);
+                }
+            }
+            for (int i = w; ok && i < sg.n; i += 2, ++kw) {
+                if (!mbar_wait_warp(&bars->p_full[w], (uint32_t)(kw & 1), abort)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const int cst = (ci0 + i) % STG;
+                const uint64_t dv = dv0 + (uint32_t)(cst * (KV_STAGE >> 4));
+                if (lead) {
 #pragma unroll
                     for (int kk = 0; kk < TT / 16; ++kk) {
                         // 16 tokens of P = 8 TMEM columns; 16 tokens of V = two 8-token groups
                         mma_bf16_ts(o_tmem, s_tmem + (uint32_t)(kk * 8),
-                                    sw128_mnmajor_desc2(V + kk * 2 * GROUP_STRIDE, HALF_STRIDE, GROUP_STRIDE),
-                                    idesc_o, (i >= 2 || kk > 0) ? 1u : 0u);
+                                    dv + (uint64_t)(kk * (2 * GROUP_STRIDE >> 4)), idesc_o,
+                                    (i >= 2 || kk > 0) ? 1u : 0u);
                     }
                     mma_commit(&bars->kv_empty[cst]);
                     mma_commit(&bars->pv_done[w]);
-                    if (i + 2 < sg.n) {
-                        // S buffer w is free: softmax i has read it (p_full above)
-                        const int cn = ci0 + i + 2;
-                        if (!mbar_wait(&bars->kv_full[cn % STG], (cn / STG) & 1, abort)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        fence_proxy_async();  // cp.async data -> tensor-core reads
-                        issue_s(cn % STG);
-                    }
                 }
-                ci0 += sg.n;
+                if (i + 2 < sg.n) {
+                    // S buffer w is free: softmax i has read it (p_full above)
+                    const int cn = ci0 + i + 2;
+                    if (!mbar_wait_warp(&bars->kv_full[cn % STG], (cn / STG) & 1, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    fence_proxy_async();  // cp.async data -> tensor-core reads
+                    issue_s(cn % STG);
+                }
             }
-            mma_commit(&bars->fin);  // completes when every MMA of this issuer is done
+            ci0 += sg.n;
         }
+        if (lead) mma_commit(&bars->fin);  // completes when every MMA of this issuer is done
         __syncwarp();
     } else if (warp < 8 && (warp & 3) < act_warps) {
         // ------------------------------------------------------------ softmax + epilogue

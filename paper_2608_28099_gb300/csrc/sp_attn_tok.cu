@@ -502,8 +502,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         bool ok = true;
         auto issue_s = [&]() {
             if (!ok || ws.done()) return;
-            if (ws.i == 0) ok = mbar_wait(&bars->q_full[rq.slot], rq.ph, abort);
-            ok = ok && mbar_wait(&bars->k_full[rk.slot], rk.ph, abort);
+            if (ws.i == 0) ok = mbar_wait_warp(&bars->q_full[rq.slot], rq.ph, abort);
+            ok = ok && mbar_wait_warp(&bars->k_full[rk.slot], rk.ph, abort);
             if (!ok) return;
             tc_fence_after();
             fence_proxy_async();  // cp.async data -> tensor-core reads
@@ -535,9 +535,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (Walk w(prefix, B, x0, x1); ok && !w.done(); w.next(), ph ^= 1) {
             const uint64_t dv = dv0 + (uint32_t)(rv.slot * (SLOT >> 4));
             const bool two = w.tiles() == 2;
-            if (!mbar_wait(&bars->v_full[rv.slot], rv.ph, abort)) break;
+            if (!mbar_wait_warp(&bars->v_full[rv.slot], rv.ph, abort)) break;
             fence_proxy_async();
-            if (!mbar_wait(&bars->p_full, ph, abort)) break;
+            if (!mbar_wait_warp(&bars->p_full, ph, abort)) break;
             tc_fence_after();
             if (lead) {
 #pragma unroll
