@@ -221,13 +221,11 @@ sp_status enqueue_attention(AttnArgs &a, void *ws, size_t ws_bytes, int attn_pat
                             cudaEvent_t *ev_attn = nullptr, cudaEvent_t *ev_merge = nullptr,
                             int seg_cost = -1, int merge_mode = 0) {
     a.tc_ctas = attn_tc_ctas(n_sm, a.Hkv);
-    a.tc_min_tiles = forced_split > 0 ? forced_split / 64 : kAttnMinTiles;
-    a.tc_seg_cost = seg_cost >= 0 ? seg_cost
-                    : a.kv.layout == SP_KV_CONTIGUOUS && !attention_tok_supported(a) ? kAttnSegCostContiguous
-                                                                                     : kAttnSegCost;
+    a.tc_seg_cost = seg_cost >= 0 ? seg_cost : kAttnSegCost;
     // few sequences over many groups: each pair has many partials, merged by a
     // kernel spread over (head, sequence, row) instead of one CTA per pair
     a.tc_merge_kernel = merge_mode == 2 || (merge_mode == 0 && 4 * a.B < a.tc_ctas / a.Hkv);
+    a.tc_min_tiles = forced_split > 0 ? forced_split / 64 : a.tc_merge_kernel ? kAttnMinTilesMerged : kAttnMinTiles;
     const size_t need = attention_workspace_bytes(a.B, a.Hkv, a.R, a.dh, a.n_splits, n_sm);
     if (ws_bytes < need) return fail(SP_ERR_INVALID_ARG, "attention workspace too small (%zu < %zu)", ws_bytes, need);
     const size_t pairs = (size_t)a.B * a.Hkv;

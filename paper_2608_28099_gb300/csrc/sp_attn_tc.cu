@@ -129,9 +129,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     // Lengths and ids come from the caller, not from the previous kernel, so
     // this runs before pdl_wait.
     int2 *seqs = (int2 *)(smem + OFF_SEQ);  // (sid, len) of sequence b
-    build_prefix<THREADS>(a, prefix, seqs, bars->wsum);
+    build_prefix<THREADS>(a, prefix, seqs, bars->wsum, blockIdx.x == 0 ? a.status : nullptr);
     const int T = prefix[B];
-    const int n_grp = min((int)gridDim.x / Hkv, ceil_div(T, max(1, a.tc_min_tiles)));
+    const int n_grp = share_count((int)gridDim.x / Hkv, T, B, a.tc_min_tiles);
     const int grp = blockIdx.x / Hkv, g = blockIdx.x - grp * Hkv;
     if (grp >= n_grp) {  // uniform over the CTA: no tile for this one
         if (threadIdx.x == 0 && a.l2_next)
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         return;
     }
     int *cuts = (int *)(smem + OFF_CUTS);
-    for (int j = threadIdx.x; j <= n_grp; j += THREADS) cuts[j] = share_start(prefix, B, T, n_grp, j, a.tc_seg_cost);
+    if (threadIdx.x < PLAN_THREADS) build_cuts(prefix, B, T, n_grp, a.tc_seg_cost, cuts, bars->wsum);
     __syncthreads();
     const int x0 = cuts[grp], x1 = cuts[grp + 1];
 
@@ -741,64 +741,64 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // Merge of the partial segments for small batches (a few long sequences, each
-// spread over many groups): one block per (kv head g, sequence b, query row),
-// one thread per dim, the pair's segments combined in the exp2 domain in
-// chunks of eight with their loads issued together.  Pairs inside one share
-// were finished by the attention kernel.
-__global__ void __launch_bounds__(DH) attn_tc_merge_kernel(AttnArgs a) {
+// spread over many groups): one block per (kv head g, sequence b, four query
+// rows), a warp per row and four dims a lane, the pair's segments combined in the
+// exp2 domain in chunks of eight with their loads issued together.  Bound by its
+// latencies (lengths, cuts, partials): the lengths are read in parallel and one
+// wave of blocks holds the work (with one row a block and the lengths read in turn,
+// attention and merge of 4 x 4000 tokens, 96 query rows, took 36 us; 26 now).
+// Pairs inside one share were finished by the attention kernel.
+constexpr int MERGE_ROWS = PLAN_THREADS / 32;
+__global__ void __launch_bounds__(PLAN_THREADS) attn_tc_merge_kernel(AttnArgs a) {
     pdl_trigger();
     __shared__ int prefix[MAX_B + 1];
     __shared__ int cuts[MAX_GRP + 1];
-    const int g = blockIdx.x, b = blockIdx.y, rr = blockIdx.z, c = threadIdx.x;
+    __shared__ int scratch[2 * MERGE_ROWS];
+    const int g = blockIdx.x, b = blockIdx.y, rr = blockIdx.z * MERGE_ROWS + (threadIdx.x >> 5);
+    const int c = (threadIdx.x & 31) * 4;
     const int B = a.B, Hkv = a.Hkv, R = a.R, k = a.k;
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int bb = 0; bb < B; ++bb) {
-            prefix[bb] = run;
-            const SeqRef sq = resolve_seq(a.seq_ids, a.seq_lens, a.lens_by_batch, bb, a.kv.n_seqs,
-                                          a.max_seq_len, nullptr);
-            run += ceil_div(sq.len + a.r0 + k, TT);
-        }
-        prefix[B] = run;
-    }
-    __syncthreads();
+    build_prefix<PLAN_THREADS>(a, prefix, nullptr, scratch, nullptr);
     const int T = prefix[B];
-    const int n_grp = min(a.tc_ctas / Hkv, ceil_div(T, max(1, a.tc_min_tiles)));
-    for (int j = threadIdx.x; j <= n_grp; j += blockDim.x) cuts[j] = share_start(prefix, B, T, n_grp, j, a.tc_seg_cost);
+    const int n_grp = share_count(a.tc_ctas / Hkv, T, B, a.tc_min_tiles);
+    build_cuts(prefix, B, T, n_grp, a.tc_seg_cost, cuts, scratch);
     __syncthreads();
     const int j0 = group_of(cuts, n_grp, prefix[b]);
     const int j1 = group_of(cuts, n_grp, prefix[b + 1] - 1);
-    if (j0 == j1) return;  // written by the attention kernel
-    pdl_wait();            // the partials come from the attention kernel
+    if (j0 == j1 || rr >= R) return;  // written by the attention kernel; no such row
+    pdl_wait();                       // the partials come from the attention kernel
     const int ns = j1 - j0 + 1;
-    float mm = -INFINITY, l = 0.f, o = 0.f;
+    float mm = -INFINITY, l = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
     for (int e0 = 0; e0 < ns; e0 += 8) {
-        float mv[8], lv[8], ov[8];
+        float2 ml[8];
+        float4 ov[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const bool in = e0 + e < ns;
-            const size_t sl = ((size_t)j0 + e0 + e + b) * Hkv + g;
-            mv[e] = in ? __ldcg(a.part_ml + (sl * R + rr) * 2) : -INFINITY;
-            lv[e] = in ? __ldcg(a.part_ml + (sl * R + rr) * 2 + 1) : 0.f;
-            ov[e] = in ? __ldcg(a.part_o + (sl * R + rr) * DH + c) : 0.f;
+            const size_t row = (((size_t)j0 + e0 + e + b) * Hkv + g) * R + rr;
+            ml[e] = in ? __ldcg((const float2 *)(a.part_ml + row * 2)) : make_float2(-INFINITY, 0.f);
+            ov[e] = in ? __ldcg((const float4 *)(a.part_o + row * DH + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         float mn = mm;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) mn = fmaxf(mn, mv[e]);
+        for (int e = 0; e < 8; ++e) mn = fmaxf(mn, ml[e].x);
         if (mn == -INFINITY) continue;
         const float al = mm == -INFINITY ? 0.f : exp2f(mm - mn);
         l *= al;
-        o *= al;
+        o.x *= al, o.y *= al, o.z *= al, o.w *= al;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const float w = mv[e] == -INFINITY ? 0.f : exp2f(mv[e] - mn);
-            l += w * lv[e];
-            o += w * ov[e];
+            const float w = ml[e].x == -INFINITY ? 0.f : exp2f(ml[e].x - mn);
+            l += w * ml[e].y;
+            o.x += w * ov[e].x, o.y += w * ov[e].y, o.z += w * ov[e].z, o.w += w * ov[e].w;
         }
         mm = mn;
     }
     const int hl = rr / k, r = rr - hl * k;
-    act_store(a.out, (((size_t)b * k + r) * a.Hq + g * a.G + hl) * DH + c, l > 0.f ? o / l : 0.f);
+    const bool any = l > 0.f;
+    act_store4(a.out, (((size_t)b * k + r) * a.Hq + g * a.G + hl) * DH + c,
+               make_float4(any ? o.x / l : 0.f, any ? o.y / l : 0.f, any ? o.z / l : 0.f, any ? o.w / l : 0.f));
 }
 
 }  // namespace
@@ -828,7 +828,7 @@ cudaError_t launch_attention_tc(const AttnArgs &a, const CUtensorMap *map_k,
                      map_v ? *map_v : dummy, a);
     }
     if (e != cudaSuccess || !a.tc_merge_kernel) return e;
-    return launch_k(attn_tc_merge_kernel, dim3(a.Hkv, a.B, a.R), dim3(DH), 0, st, a);
+    return launch_k(attn_tc_merge_kernel, dim3(a.Hkv, a.B, ceil_div(a.R, MERGE_ROWS)), dim3(PLAN_THREADS), 0, st, a);
 }
 
 }  // namespace sp

@@ -1,7 +1,7 @@
 // Split-KV attention of the k appended rows over [cached ; new] keys
 // (Sec. 3.3, Eq. 1-3) on tcgen05 tensor cores with the tokens on the MMA's M
-// side, for head_dim 128 and bf16 caches: the kernel for up to 64 query rows per kv
-// head, or 80 plain ones (tok_layout below).
+// side, for head_dim 128 and bf16 caches: the kernel for up to 32 query rows per kv
+// head, and for up to 80 where there is enough to stream (tok_wins below).
 //
 // The work list, its cuts and the partials are those of sp_attn_tc.cu: CTA
 // (j, g) attends kv head g over share j of the 64-token tile list; a share's
@@ -262,20 +262,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     const bool paged = a.kv.layout == SP_KV_PAGED;
     pdl_trigger();
 
-    build_prefix<THREADS>(a, prefix, seqs, bars->wsum);
+    build_prefix<THREADS>(a, prefix, seqs, bars->wsum, blockIdx.x == 0 ? a.status : nullptr);
     const int T = prefix[B];
-    const int n_grp = min((int)gridDim.x / Hkv, ceil_div(T, max(1, a.tc_min_tiles)));
+    const int n_grp = share_count((int)gridDim.x / Hkv, T, B, a.tc_min_tiles);
     const int grp = blockIdx.x / Hkv, g = blockIdx.x - grp * Hkv;
     if (grp >= n_grp) {  // uniform over the CTA: no tile for this one
         if (threadIdx.x == 0 && a.l2_next)
             prefetch_l2_share(a.l2_next, a.l2_next_bytes, blockIdx.x, gridDim.x);
         return;
     }
-#pragma unroll 1
-    for (int j = threadIdx.x; j <= n_grp; j += THREADS / 4) {
-        if (threadIdx.x >= THREADS / 4) break;  // (set-up is shared out over the warps)
-        cuts[j] = share_start(prefix, B, T, n_grp, j, a.tc_seg_cost);
-    }
+    if (threadIdx.x < PLAN_THREADS)  // (set-up is shared out over the warps)
+        build_cuts(prefix, B, T, n_grp, a.tc_seg_cost, cuts, bars->wsum);
     if (threadIdx.x >= 128 && threadIdx.x < 256) {
         const int rr = threadIdx.x - 128;
         const int rk = rr % k;
@@ -846,22 +843,34 @@ __global__ void __launch_bounds__(THREADS, 1)
 // then the rings (K in front of V).
 // Its cost grows with the query rows (scores a thread, the queries' and P's
 // shared memory) where the queries-on-M kernel of sp_attn_tc.cu pays for 128 rows
-// always.  Attention step, that kernel -> this one, d = 4096 heads:
-//   up to 48 rows: every shape 1.06-1.7x (B = 200, L = 100..300: 93 -> 56 us at 4
-//     rows, 107 -> 100 at 48; B = 40, L = 200..3000: 77 -> 55 and 80 -> 68 us);
-//   64 rows plain: 1.0-1.2x (B = 200, L = 1000..1500: 275 -> 232 us); hi + lo
-//     228 -> 199 us at B = 64, L = 1000..8000, but 113 -> 121 at L = 100..300;
-//   80 rows plain: contiguous 389 -> 349 us (B = 16, L = 30000), paged 326 -> 316,
-//     303 -> 275 (B = 200, L = 1000..1500) and 167 -> 158 (L = 100..300), but 34 ->
-//     35 (B = 4, L = 8000) and 84 -> 86 (B = 40, L = 200..3000);
-//   96 and 128 rows plain, 80 hi + lo: slower (140 -> 240 us at 96 rows, L = 100..300).
+// always; its segments cost less, so it needs work to stream.  Attention step, that
+// kernel -> this one in us, d = 4096 heads (8 kv heads), contiguous / paged:
+//   up to 32 rows: everywhere (B = 200, L = 100..300: 93 -> 56 at 4 rows);
+//   48 rows: B = 40, L = 300..500 50 -> 40 / 46 -> 38, B = 200, L = 1000..1500 251 ->
+//     230 / 245 -> 212, B = 8, L = 32000 184 -> 181 / 171 -> 169; but 16 x 500 16.8 ->
+//     17.1 and 4 x 1000 15.2 -> 17.6;
+//   64 rows plain: B = 40, L = 200..3000 79 -> 78 / 72 -> 69, B = 100 158 -> 152 / 147 ->
+//     136, 16 x 8000 contiguous 112 -> 108; but 16 x 500 22 -> 28 / 20 -> 27;
+//   64 rows hi + lo: paged, B = 100, L = 200..3000 148 -> 137, 8 x 4000 42 -> 39, 16 x
+//     8000 contiguous 104 -> 101; but B = 40, L = 200..3000 contiguous 78 -> 80, and
+//     B = 200, L = 100..300 112 -> 121 / 111 -> 119;
+//   80 rows plain: long contiguous caches only (16 x 30000 392 -> 349, 8 x 32000 211 ->
+//     198; paged 168 -> 176, B = 40, L = 200..3000 88 -> 95 / 76 -> 86).
+//   96 and 128 rows plain, 80 hi + lo: slower (140 -> 240 at 96 rows, L = 100..300).
+bool tok_wins(const AttnArgs &a, int R16) {
+    const bool paged = a.kv.layout == SP_KV_PAGED;
+    const long long tokens = (long long)a.B * a.max_seq_len;
+    const bool long_contiguous = !paged && a.max_seq_len > 4096 && tokens >= 100 * 1024;
+    if (R16 <= 32) return true;
+    if (R16 <= 48) return tokens >= 16 * 1024;
+    if (R16 <= 64 && a.tc_q_plain) return long_contiguous || 2ll * a.B * a.Hkv >= 3ll * a.tc_ctas;
+    if (R16 <= 64) return paged ? a.max_seq_len > 512 && tokens >= 32 * 1024 : long_contiguous;
+    return R16 <= 80 && a.tc_q_plain && long_contiguous;
+}
+
 bool tok_layout(const AttnArgs &a, TokLayout *lay) {
     const int R16 = (a.R + 15) / 16 * 16;
-    if (R16 > (a.tc_q_plain ? 80 : 64)) return false;
-    if (R16 == 64 && !a.tc_q_plain && a.max_seq_len <= 512) return false;
-    if (R16 == 80 && a.kv.layout == SP_KV_PAGED && a.max_seq_len > 512 &&
-        (long long)a.B * a.max_seq_len < 160 * 1024)
-        return false;
+    if (!tok_wins(a, R16)) return false;
     const int tab = ((a.B + 2) & ~1) * 4 + a.B * 8;
     const int front = (OFF_TAB + tab + 1023) & ~1023;
     const int q = R16 * 256 * (a.tc_q_plain ? 1 : 2), p = STEP * 128 * ((R16 + 63) / 64);

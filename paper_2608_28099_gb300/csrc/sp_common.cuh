@@ -225,16 +225,20 @@ void plan_attention(int B, int Hkv, int k, int max_seq_len, int forced_split, in
 // part_ml) sized for either kernel: B Hkv n_splits units (CUDA cores) or
 // attn_tc_ctas(n_sm, Hkv) + B Hkv slots (tensor cores).
 size_t attention_workspace_bytes(int B, int Hkv, int R, int dh, int n_splits, int n_sm);
-// Default fewest tiles per CTA of the tensor-core kernel (64 tokens each).
+// Default fewest 64-token tiles per share of the tensor-core kernels: fewer where a
+// kernel of its own merges the partials (few sequences), since a partial then costs
+// less than the merge inside.  Attention step at 4 / 8 tiles, paged, 16 and 96 query
+// rows: one sequence of 1200 tokens 9.0 / 10.9 and 15.8 / 17.2 us, two of 600 10.1 /
+// 12.2 and 16.5 / 22.6; merged inside, eight of 600 14.4 / 11.4 and 20.7 / 21.0.
+constexpr int kAttnMinTilesMerged = 4;
 constexpr int kAttnMinTiles = 8;
-// Default cost of a segment boundary in the tensor-core kernels, in 64-token
+// Default cost of a segment in the tensor-core kernels, in 64-token
 // tiles (the epilogue, the first step's row maxima, a merge at a share's end).
 // Tokens-on-M kernel, attention of 4B (contiguous) / 8B paged / 27B long in us:
-// 24.8, 207, 182 at 4; 22.8, 202, 178 at 12; 25.0, 210, 182 at 28.
+// 24.8, 207, 182 at 4; 22.8, 202, 178 at 12; 25.0, 210, 182 at 28.  Queries-on-M
+// kernel, contiguous, 96 rows at 12 / 28: 8 x 3000 tokens 42.8 / 49.5, 24 x 1000
+// 50.2 / 58.1, 40 x 3000 135.2 / 135.6.
 constexpr int kAttnSegCost = 12;
-// Queries-on-M kernel, contiguous caches (cp.async tiles, 4B shape): 40.5 us at
-// 28 against 42.6 at 12.
-constexpr int kAttnSegCostContiguous = 28;
 // Persistent CTAs of the tensor-core kernel: whole groups of Hkv (one CTA per
 // kv head), as many groups as the SMs hold, at least one.
 inline int attn_tc_ctas(int n_sm, int Hkv) { return (n_sm / Hkv > 1 ? n_sm / Hkv : 1) * Hkv; }

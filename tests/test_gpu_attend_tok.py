@@ -86,3 +86,54 @@ def test_plain_queries_through_classify(hq, k, T, layout):
         run = GpuRun(w)
         compare(run.logits(), oracle_logits(w), label=f"plain R={hq * k}")
     run.close()
+
+
+def _lens(B, longest):
+    lens = np.random.default_rng(B).integers(0, 200, B)
+    lens[B // 2] = longest
+    return [int(x) for x in lens]
+
+
+# the row counts that take this kernel only from some size on: many sequences (64
+# rows plain), long contiguous caches (64 and 80 rows plain)
+@pytest.mark.parametrize("hq,k,layout,B,longest", [
+    (4, 16, wl.LAYOUT_PAGED, 120, 200), (4, 15, wl.LAYOUT_CONTIGUOUS, 115, 129),
+    (4, 16, wl.LAYOUT_CONTIGUOUS, 25, 4200), (5, 16, wl.LAYOUT_CONTIGUOUS, 25, 4200),
+])
+def test_plain_queries_from_a_size_on(hq, k, layout, B, longest):
+    w = wl.custom(wl.Shape(256, 2 * hq, 2, 128, 512, k, 2), _lens(B, longest), layout, 730 + k, rows_per_seq=True)
+    run = GpuRun(w)
+    compare(run.logits(), oracle_logits(w), label=f"plain R={hq * k}")
+    run.close()
+
+
+@pytest.mark.parametrize("k,page,B,longest", [(12, 0, 8, 2100), (16, 16, 16, 2100), (16, 0, 25, 4200)])
+def test_exact_queries_from_a_size_on(k, page, B, longest):
+    ensure_built()
+    shape = wl.Shape(256, 8, 2, 128, 256, k, 2, page_size=page or 16)
+    w = wl.custom(shape, _lens(B, longest), wl.LAYOUT_PAGED if page else wl.LAYOUT_CONTIGUOUS, 740 + k)
+    rng = np.random.default_rng(k)
+    q = rng.standard_normal((B, k, 8, 128)).astype(np.float32)
+    kn, vn = (rng.standard_normal((B, k, 2, 128)).astype(np.float32) for _ in range(2))
+    ref = so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn)))
+    out, _ = _attend(shape, w, q, kn, vn, 2)
+    # as above: bf16 new values and scores, 2e-2 in all at 1.5 times these queries
+    assert np.all(np.abs(out - ref) <= 2e-2 * (1 + np.abs(ref)))
+
+
+# shares: whole sequences in a share each, more sequences than shares hold, one
+# sequence over many shares, empty caches
+@pytest.mark.parametrize("lens", [[500] * 16, [300] * 3, [1000] * 80 + [0] * 9, [0] * 30 + [5000], [2000, 70, 0, 70]])
+@pytest.mark.parametrize("hq,k", [(4, 4), (6, 16)])
+def test_shares(lens, hq, k):
+    ensure_built()
+    shape = wl.Shape(256, 4 * hq, 4, 128, 256, k, 2)
+    w = wl.custom(shape, lens, wl.LAYOUT_PAGED, 750 + len(lens))
+    rng = np.random.default_rng(len(lens))
+    B = len(lens)
+    q = rng.standard_normal((B, k, 4 * hq, 128)).astype(np.float32)
+    kn, vn = (rng.standard_normal((B, k, 4, 128)).astype(np.float32) for _ in range(2))
+    ref = so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn)))
+    for _ in range(2):  # the merge counters are clear again after the first call
+        out, _ = _attend(shape, w, q, kn, vn, 2)
+        assert np.all(np.abs(out - ref) <= 2e-2 * (1 + np.abs(ref)))
