@@ -253,10 +253,8 @@ enum {
     SP_OPT_ATTN_SEG_COST = 6, /* tensor-core attention: the cost of a segment
                                  boundary, in 64-token tiles, that the cuts
                                  between CTA shares balance (-1..1024); -1 = the
-                                 built-in default (12; 28 for a contiguous cache
-                                 with more than 96 hi + lo query rows per kv
-                                 head).  Changes the work split only, never the
-                                 result beyond rounding order                    */
+                                 built-in default (12).  Changes the work split
+                                 only, never the result beyond rounding order    */
     SP_OPT_ACT_PRECISION = 7, /* activations fed to the tensor-core
                                  projections: 0 = automatic (gate/up and down
                                  take plain bf16 when pool is SP_POOL_MEAN and

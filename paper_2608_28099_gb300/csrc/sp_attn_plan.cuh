@@ -242,10 +242,11 @@ __device__ __forceinline__ void build_prefix(const AttnArgs &a, int *prefix, int
 // contiguous bytes per plane.  Loads through registers would need a
 // dependent round trip per two segments, each waiting behind the other
 // SMs' cache streams.
-// (own: a segment already in place, or -1.  Run by all THREADS threads; good: every wait of the kernel was served; uniform over the CTA.)
+// (Run by all THREADS threads; good: every wait of the kernel was served; uniform
+// over the CTA.)
 template <int THREADS>
 __device__ __forceinline__ void staged_merge(const AttnArgs &a, uint8_t *stage, int b, int g, int n_seg,
-                                             size_t slot0, bool good, int own = -1) {
+                                             size_t slot0, bool good) {
     const int R = a.R, k = a.k, Hkv = a.Hkv;
     __threadfence();            // the other segments' partials are read after their count
     float2 *st_ml = (float2 *)(stage + (size_t)n_seg * R * DH * 4);
@@ -253,13 +254,12 @@ __device__ __forceinline__ void staged_merge(const AttnArgs &a, uint8_t *stage, 
 #pragma unroll 4
     for (int idx = threadIdx.x; idx < n_seg * units; idx += THREADS) {
         const int e = idx / units, rem = idx - e * units;
-        if (e != own)
-            cp_async16(stage + (size_t)idx * 16, a.part_o + (slot0 + (size_t)e * Hkv) * R * DH + (size_t)rem * 4);
+        cp_async16(stage + (size_t)idx * 16, a.part_o + (slot0 + (size_t)e * Hkv) * R * DH + (size_t)rem * 4);
     }
 #pragma unroll 1
     for (int idx = threadIdx.x; idx < n_seg * R; idx += THREADS) {
         const int e = idx / R, rr = idx - e * R;
-        if (e != own) st_ml[idx] = __ldcg((const float2 *)(a.part_ml + ((slot0 + (size_t)e * Hkv) * R + rr) * 2));
+        st_ml[idx] = __ldcg((const float2 *)(a.part_ml + ((slot0 + (size_t)e * Hkv) * R + rr) * 2));
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();

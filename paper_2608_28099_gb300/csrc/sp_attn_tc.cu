@@ -5,7 +5,7 @@
 // Work balance: the keys of every sequence b are cut into 64-token tiles, and
 // the tiles of all sequences, in order, form one list of T tiles per kv head.
 // The persistent grid holds n groups of Hkv CTAs (n Hkv <= SMs); CTA (j, g)
-// attends kv head g over the equal share [j T / n, (j+1) T / n) of the list,
+// attends kv head g over share j of the list (about T / n tiles: sp_attn_plan.cuh),
 // whatever the mix of lengths, so a ragged batch keeps every SM streaming
 // until the end, and the Hkv heads of a token range are read at the same time
 // (a token's keys of all heads sit together in the cache: whole cache rows or
