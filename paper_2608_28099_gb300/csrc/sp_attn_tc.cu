@@ -764,8 +764,11 @@ __global__ void __launch_bounds__(PLAN_THREADS) attn_tc_merge_kernel(AttnArgs a)
     __syncthreads();
     const int j0 = group_of(cuts, n_grp, prefix[b]);
     const int j1 = group_of(cuts, n_grp, prefix[b + 1] - 1);
+    // The partials come from the attention kernel.  Blocks without a merge wait too:
+    // where no pair is split this grid would else be done before the attention, and
+    // the next kernel waits for this grid only.
+    pdl_wait();
     if (j0 == j1 || rr >= R) return;  // written by the attention kernel; no such row
-    pdl_wait();                       // the partials come from the attention kernel
     const int ns = j1 - j0 + 1;
     float mm = -INFINITY, l = 0.f;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -1,0 +1,58 @@
+"""Order of dependent kernels (no GPU): every kernel is launched with programmatic
+stream serialisation, so what keeps the stream's order is where each kernel calls
+pdl_wait() and pdl_trigger().  A wrong place shows only as a rare race, so the
+sources are checked: by kernel, the statements in front of the first wait."""
+import glob
+import os
+import re
+
+import pytest
+
+from conftest import ROOT
+
+CSRC = os.path.join(ROOT, "paper_2608_28099_gb300", "csrc")
+
+
+def _kernels():
+    """name -> body of every __global__ function, comments removed."""
+    out = {}
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        with open(path) as f:
+            s = re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", f.read(), flags=re.S))
+        for m in re.finditer(r"__global__\s+void\b.*?(\w+)\s*\((?=\s*(?:const\s+)?(?:__grid_constant__|"
+                             r"T\b|TX\b|float\b|float4\b|PartIn\b|QkvRopeArgs\b|AttnArgs\b|CUtensorMap\b))", s, flags=re.S):
+            i = s.index("{", m.end())
+            depth, j = 1, i + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(s[j], 0)
+                j += 1
+            out[m.group(1)] = s[i:j]
+    return out
+
+
+KERNELS = _kernels()
+
+# Blocks that may leave before the wait, since others of the same grid always wait
+# (a grid is complete only when all of its blocks are).
+LEAVES_EARLY = {
+    "attn_tc_kernel": "groups past the last share; group 0 has one",
+    "attn_tok_kernel": "groups past the last share; group 0 has one",
+    "attn_split_simt": "units past the sequence's end; unit 0 never is (k >= 1 new rows)",
+}
+
+
+def test_every_kernel_is_found():
+    with_launch = set()
+    for path in glob.glob(os.path.join(CSRC, "*.cu")):
+        with open(path) as f:
+            with_launch |= set(re.findall(r"launch_k\(\s*(\w+)", f.read()))
+    assert with_launch == set(KERNELS)
+
+
+@pytest.mark.parametrize("name", sorted(KERNELS))
+def test_a_grid_completes_after_the_one_before_it(name):
+    body = KERNELS[name]
+    assert "pdl_wait()" in body, "a grid that never waits may complete before the one in front of it"
+    before = body[:body.index("pdl_wait()")]
+    if name not in LEAVES_EARLY:
+        assert not re.search(r"\breturn\b", before), "a block leaves before the wait"
