@@ -1043,6 +1043,7 @@ sp_status sp_attend(sp_stream stream, const sp_attn_dims *dm, int batch, const i
     a.kv = to_dev(kv);
     a.q = d_q; a.k_new = d_k_new; a.v_new = d_v_new;
     a.status = d_status;
+    a.first = 1;  // (on the tensor path a memset is in front of the attention)
     a.gathered = d_gathered_pages;
     a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)a.dh));
     a.out.f32 = out_dtype == SP_F32 ? (float *)d_out : nullptr;

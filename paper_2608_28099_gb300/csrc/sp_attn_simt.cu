@@ -55,6 +55,7 @@ __device__ __forceinline__ long long cache_offset(const KVDev &kv, int sid, int 
 
 template <typename TKV, int DH>
 __global__ void __launch_bounds__(kThreads) attn_split_simt(AttnArgs a) {
+    if (a.first) pdl_wait();
     pdl_trigger();
     extern __shared__ float smem[];
     const int s = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(kThreads) attn_split_simt(AttnArgs a) {
     // first is stored, the next tile's during this one's products (a chain of
     // round trips: the tiny layer's step took 11.3 us with element loads in turn, 7.6 now).  The cache is the caller's: the first tile is requested
     // before the previous kernel (which writes the queries and new rows) is done,
-    // unless it holds new rows.
+    // unless it holds new rows (or there is no kernel of this call in front).
     constexpr int NV = kTile * DH / 4 / kThreads;
     float4 kr[NV], vr[NV];
     int bad = 0;

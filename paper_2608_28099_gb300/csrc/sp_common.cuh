@@ -28,6 +28,12 @@ template <> __device__ __forceinline__ bf16 from_f<bf16>(float x) { return __flo
 // visible; every kernel calls it before touching data an earlier kernel
 // writes, and before writing scratch an earlier kernel may still read.
 // pdl_trigger() allows the next kernel to launch (it still waits in pdl_wait).
+// Inputs of the caller (ids, lengths, page table, cache, sp_project's weights) are
+// read in front of the wait by kernels behind the first one of a call.  So the
+// first kernel of a call waits before it reads any of them and triggers only after
+// that: everything behind it starts when the caller's earlier work on the stream,
+// which may itself trigger early (sp_project writing a cache), is complete.  A
+// kernel that can be the first one takes that from its arguments, or always does so.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -211,6 +217,7 @@ struct AttnArgs {
     int *counters;                // [B][Hkv] finished segments, zero before the launch (tensor
                                   // cores: the last segment of a pair merges it)
     int *status;
+    int first;                    // CUDA cores: 1 = the first kernel of the call (see pdl_wait)
     int *gathered;                // [B][max_pages] or NULL
     float scale_log2;             // log2(e) / sqrt(dh)
     ActOut out;                   // merge output [B][k][Hq][dh]

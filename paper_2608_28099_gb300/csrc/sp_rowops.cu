@@ -34,8 +34,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) rmsnorm_rows_loop_kernel(const T *__restrict__ x, int row_mod,
                                                            const float *__restrict__ gain, float eps,
                                                            int d, ActOut out) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // a call's first kernel: after the wait
     __shared__ float red[32];
     const int m = blockIdx.x;
     const T *xr = x + (size_t)(row_mod ? m % row_mod : m) * d;
@@ -71,6 +71,8 @@ __global__ void __launch_bounds__(256) rmsnorm_rows_loop_kernel(const T *__restr
 // take one pass.
 template <int TPB>
 __global__ void __launch_bounds__(TPB) qkv_rope_kernel(QkvRopeArgs a) {
+    const bool first = a.shared;  // the shared prompt's projections are the handle's
+    if (first) pdl_wait();
     pdl_trigger();
     __shared__ int s_pos;
     const int m = blockIdx.x;
@@ -80,7 +82,7 @@ __global__ void __launch_bounds__(TPB) qkv_rope_kernel(QkvRopeArgs a) {
                                      a.max_seq_len, a.status);
         s_pos = s.len + a.r0 + (a.k_task ? r % a.k_task : r);
     }
-    pdl_wait();
+    if (!first) pdl_wait();
     if (a.zero_ints && m == 0)
         for (int t = threadIdx.x; t < a.n_zero; t += blockDim.x) a.zero_ints[t] = 0;
     __syncthreads();
@@ -135,6 +137,8 @@ __global__ void __launch_bounds__(TPB) qkv_rope_kernel(QkvRopeArgs a) {
 
 // The same with 256 threads and one item per loop step (many rows).
 __global__ void __launch_bounds__(256) qkv_rope_rows_kernel(QkvRopeArgs a) {
+    const bool first = a.shared;  // the shared prompt's projections are the handle's
+    if (first) pdl_wait();
     pdl_trigger();
     __shared__ int s_pos;
     const int m = blockIdx.x;
@@ -144,7 +148,7 @@ __global__ void __launch_bounds__(256) qkv_rope_rows_kernel(QkvRopeArgs a) {
                                      a.max_seq_len, a.status);
         s_pos = s.len + a.r0 + (a.k_task ? r % a.k_task : r);
     }
-    pdl_wait();
+    if (!first) pdl_wait();
     if (a.zero_ints && m == 0)
         for (int t = threadIdx.x; t < a.n_zero; t += blockDim.x) a.zero_ints[t] = 0;
     __syncthreads();
@@ -257,7 +261,6 @@ template <typename T, int V, int TPB>  // V: 4-element chunks per thread, d <= 4
 __global__ void __launch_bounds__(TPB) rmsnorm_rows_kernel(const T *__restrict__ x, int row_mod,
                                                                     const float *__restrict__ gain,
                                                                     float eps, int d, ActOut out) {
-    pdl_trigger();
     __shared__ float red[TPB / 32];
     const int m = blockIdx.x, nch = d >> 2;
     float4 gv[V];
@@ -267,6 +270,7 @@ __global__ void __launch_bounds__(TPB) rmsnorm_rows_kernel(const T *__restrict__
         gv[i] = c < nch ? *(const float4 *)(gain + c * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     pdl_wait();
+    pdl_trigger();  // a call's first kernel: after the wait
     const T *xr = x + (size_t)(row_mod ? m % row_mod : m) * d;
     float4 v[V];
     float ss = 0.f;
@@ -536,8 +540,8 @@ cudaError_t launch_readout_t(int B, int d, cudaStream_t st, Args... args) {
 
 // n4 vectors of four values.
 __global__ void to_act_kernel(const float4 *__restrict__ x, size_t n4, ActOut out) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // a call's first kernel: after the wait
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4;
          i += (size_t)gridDim.x * blockDim.x)
         act_store4(out, 4 * i, x[i]);

@@ -8,7 +8,7 @@ import pytest
 import oracle.sp_oracle as so
 import paper_2608_28099_gb300 as sp
 from paper_2608_28099_gb300 import workloads as wl
-from gpu_util import GpuRun, compare, rows_tensor
+from gpu_util import GpuRun, compare, ensure_built, rows_tensor, torch_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +47,51 @@ def _classify_in_a_row(w, options=None, repeats=4):
 def test_classify(lens, hq, k):
     sh = wl.Shape(256, 2 * hq, 2, 128, 512, k, 3)
     _classify_in_a_row(wl.custom(sh, lens, wl.LAYOUT_PAGED, 900 + len(lens), rows_per_seq=True))
+
+
+@pytest.mark.parametrize("dh,kv", [(32, wl.BF16), (64, wl.F32), (128, wl.F32)])
+def test_classify_with_cuda_core_attention(dh, kv):
+    sh = wl.Shape(256, 8, 2, dh, 512, 5, 3, kv_dtype=kv)
+    _classify_in_a_row(wl.custom(sh, [250, 31, 0, 700], wl.LAYOUT_CONTIGUOUS, 920 + dh, rows_per_seq=True))
+
+
+@pytest.mark.parametrize("lens", [[24, 7], [40, 300, 1]])
+def test_attend_reads_a_cache_that_the_call_before_it_writes(lens):
+    # sp_project writes the fp32 values of a contiguous cache ([tokens][Hkv dh]) in
+    # place, sp_attend reads them: other values in every turn
+    ensure_built()
+    torch = torch_dev()
+    hkv, G, dh, k, K = 4, 2, 32, 3, 1024
+    N, M = hkv * dh, sum(lens)
+    rng = np.random.default_rng(M)
+    shape = wl.Shape(256, hkv * G, hkv, dh, 256, k, 2, kv_dtype=wl.F32)
+    w = wl.custom(shape, lens, wl.LAYOUT_CONTIGUOUS, 940)
+    wbits = wl.f32_to_bf16_bits((0.05 * rng.standard_normal((N, K))).astype(np.float32))
+    wt = torch.from_numpy(wbits.view(np.int16)).cuda()
+    wf = wl.bf16_bits_to_f32(wbits).astype(np.float64)
+    xs = [rng.standard_normal((M, K)).astype(np.float32) for _ in range(3)]
+    q = rng.standard_normal((len(lens), k, hkv * G, dh)).astype(np.float32)
+    kn, vn = (rng.standard_normal((len(lens), k, hkv, dh)).astype(np.float32) for _ in range(2))
+    cache = sp.DeviceCache(w.cache)
+    values = cache.v_flat
+    assert tuple(values.shape) == (M, hkv, dh) and values.dtype == torch.float32
+    refs = []
+    for x in xs:
+        w.cache.v_flat = (x.astype(np.float64) @ wf.T).reshape(M, hkv, dh).astype(np.float32)
+        refs.append(so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn))))
+    dims = sp.sp_attn_dims(hkv * G, hkv, dh, k, sp.SP_F32, max(lens), 0, 0)
+    ws = torch.empty(sp.sp_attend_workspace_bytes(dims, len(lens)), dtype=torch.uint8, device="cuda")
+    pws = torch.empty(max(256, sp.sp_project_workspace_bytes(M, N, K)), dtype=torch.uint8, device="cuda")
+    x_d = [torch.from_numpy(x).cuda() for x in xs]
+    q_d, kn_d, vn_d = (torch.from_numpy(t).cuda() for t in (q, kn, vn))
+    outs = [torch.empty(q.shape, device="cuda") for _ in range(60)]
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    for i, o in enumerate(outs):
+        path = 1 + (i // 3) % 2  # the projection on CUDA cores and on tensor cores in turn
+        sp.sp_project(st, M, N, K, x_d[i % 3], wt, values, path, pws, pws.numel())
+        sp.sp_attend(st, dims, len(lens), None, cache.seq_lens, cache.desc, q_d, kn_d, vn_d, o, sp.SP_F32, ws, ws.numel())
+    st.synchronize()
+    for i, o in enumerate(outs):
+        # values off by up to 4e-5 of the largest (hi + lo inputs, K = 1024), the rest fp32
+        np.testing.assert_allclose(o.cpu().numpy(), refs[i % 3], rtol=1e-3, atol=1e-3)

@@ -56,3 +56,27 @@ def test_a_grid_completes_after_the_one_before_it(name):
     before = body[:body.index("pdl_wait()")]
     if name not in LEAVES_EARLY:
         assert not re.search(r"\breturn\b", before), "a block leaves before the wait"
+
+
+# The kernels that can be the first of a public call: per-sequence rows and hidden
+# states start with the input norm, the shared prompt with the rotation, sp_attend on
+# CUDA cores with the split kernel (on tensor cores a memset is in front), sp_project
+# with the conversion of X or, on CUDA cores, with its only kernel.
+FIRST = ["rmsnorm_rows_kernel", "rmsnorm_rows_loop_kernel", "qkv_rope_kernel", "qkv_rope_rows_kernel",
+         "attn_split_simt", "to_act_kernel"]
+ALONE = ["gemm_simt_kernel", "gemv_simt_kernel"]
+
+
+@pytest.mark.parametrize("name", FIRST)
+def test_a_first_kernel_triggers_after_its_wait(name):
+    # kernels behind it read the caller's ids, lengths, page table, cache and weights
+    # in front of their own waits
+    body = KERNELS[name]
+    assert body.index("pdl_wait()") < body.index("pdl_trigger()")
+
+
+@pytest.mark.parametrize("name", FIRST + ALONE)
+def test_a_first_kernel_reads_the_callers_data_after_its_wait(name):
+    before = KERNELS[name]
+    before = before[:before.index("pdl_wait()")]
+    assert not re.search(r"resolve_seq|load_tile\(|load4\(|load8\(|\bx\[|\bX\[|\bW\[|xr\b", before)
