@@ -1,7 +1,7 @@
 // Split-KV attention of the k appended rows over [cached ; new] keys
 // (Sec. 3.3, Eq. 1-3) on tcgen05 tensor cores with the tokens on the MMA's M
 // side, for head_dim 128 and bf16 caches: the kernel for up to 32 query rows per kv
-// head, and for up to 80 where there is enough to stream (tok_wins below).
+// head, and for up to 64 in larger batches (tok_wins below).
 //
 // The work list, its cuts and the partials are those of sp_attn_tc.cu: CTA
 // (j, g) attends kv head g over share j of the 64-token tile list; a share's
@@ -64,7 +64,6 @@ constexpr int BAR_SOFT = 1, BAR_Q = 4;  // (BAR_SOFT + 1, + 2: one softmax group
 // rings, so that nothing the MMAs read past a buffer's rows leaves the window.
 struct TokLayout {
     int r16;        // query rows padded to a multiple of 16
-    int nq;         // query buffers (2, or 1 where two would cost ring slots)
     int nk, nv;     // ring slots
     int off_q, q_bytes, off_p, off_k, off_v;
     int smem;
@@ -240,7 +239,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr int EC = W < 16 ? W : 16;          // rows of an epilogue chunk
     constexpr uint32_t S_COLS = (NR + 31) / 32 * 32;  // TMEM columns of a score buffer
     constexpr uint32_t O_COL = 2 * S_COLS;
-    constexpr uint32_t TMEM_COLS = NR <= 32 ? 128 : NR <= 64 ? 256 : 512;
+    constexpr uint32_t TMEM_COLS = NR <= 32 ? 128 : 256;
+    static_assert(NR % 16 == 0 && NR <= 64, "query rows");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     TokBars *bars = (TokBars *)(smem + OFF_BAR);
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // else to do then)
         const int qt = threadIdx.x - Q_WARP * 32;
         pdl_wait();  // the rotated queries come from the previous kernel
-        Ring rg(lay.nq);
+        Ring rg(2);
         bool first = true;
 #pragma unroll 1
         for (int x = x0; x < x1;) {
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t q_step = (uint32_t)lay.q_bytes >> 4;
         const bool q_lo = !a.tc_q_plain;
         Walk ws(prefix, B, x0, x1);
-        Ring rk(lay.nk), rv(lay.nv), rq(lay.nq);
+        Ring rk(lay.nk), rv(lay.nv), rq(2);
         uint32_t sbuf = 0;
         bool ok = true;
         auto issue_s = [&]() {
@@ -839,33 +839,25 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (warp == MMA_W) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// Whether this kernel takes the call, and its shared memory: query buffers, P,
+// Whether this kernel takes the call, and its shared memory: two query buffers, P,
 // then the rings (K in front of V).
 // Its cost grows with the query rows (scores a thread, the queries' and P's
 // shared memory) where the queries-on-M kernel of sp_attn_tc.cu pays for 128 rows
-// always; its segments cost less, so it needs work to stream.  Attention step, that
-// kernel -> this one in us, d = 4096 heads (8 kv heads), contiguous / paged:
-//   up to 32 rows: everywhere (B = 200, L = 100..300: 93 -> 56 at 4 rows);
-//   48 rows: B = 40, L = 300..500 50 -> 40 / 46 -> 38, B = 200, L = 1000..1500 251 ->
-//     230 / 245 -> 212, B = 8, L = 32000 184 -> 181 / 171 -> 169; but 16 x 500 16.8 ->
-//     17.1 and 4 x 1000 15.2 -> 17.6;
-//   64 rows plain: B = 40, L = 200..3000 79 -> 78 / 72 -> 69, B = 100 158 -> 152 / 147 ->
-//     136, 16 x 8000 contiguous 112 -> 108; but 16 x 500 22 -> 28 / 20 -> 27;
-//   64 rows hi + lo: paged, B = 100, L = 200..3000 148 -> 137, 8 x 4000 42 -> 39, 16 x
-//     8000 contiguous 104 -> 101; but B = 40, L = 200..3000 contiguous 78 -> 80, and
-//     B = 200, L = 100..300 112 -> 121 / 111 -> 119;
-//   80 rows plain: long contiguous caches only (16 x 30000 392 -> 349, 8 x 32000 211 ->
-//     198; paged 168 -> 176, B = 40, L = 200..3000 88 -> 95 / 76 -> 86).
-//   96 and 128 rows plain, 80 hi + lo: slower (140 -> 240 at 96 rows, L = 100..300).
+// always, and most so for short sequences, whose steps are all first ones.  Lengths
+// are known on the device only and max_seq_len may be far above them, so the rule
+// uses the rows and the batch: it takes what no length makes more than 2 % slower.
+// Whole calls of the 8B layer in us, that kernel -> this one, paged, per-sequence rows,
+// 120 / 500 / 2000 / 4000 tokens (152 SMs, 8 kv heads):
+//   up to 32 rows: everywhere (attention alone, B = 200, L = 100..300: 93 -> 56);
+//   48 rows: B = 128 586 -> 583, 614 -> 593, 728 -> 705, 861 -> 847; B = 64 309 -> 311,
+//     327 -> 317, 379 -> 361, 465 -> 442; but B = 16, 300 to 1700 tokens 174 -> 179;
+//   64 rows: B = 128 715 -> 730, 747 -> 737, 854 -> 850, 990 -> 980; B = 64 378 -> 376,
+//     397 -> 399, 442 -> 435, 510 -> 507; but B = 32 222 -> 227, 231 -> 236, 264 -> 263,
+//     302 -> 297, and B = 16, 300 to 1700 tokens 170 -> 188; with hi + lo queries
+//     B = 128 682 -> 670 at 60 tokens, 722 -> 711 at 300, 753 -> 746 at 1000;
+//   80 rows: B = 128 968 -> 982, 1003 -> 1000, 1104 -> 1097, 1232 -> 1245.
 bool tok_wins(const AttnArgs &a, int R16) {
-    const bool paged = a.kv.layout == SP_KV_PAGED;
-    const long long tokens = (long long)a.B * a.max_seq_len;
-    const bool long_contiguous = !paged && a.max_seq_len > 4096 && tokens >= 100 * 1024;
-    if (R16 <= 32) return true;
-    if (R16 <= 48) return tokens >= 16 * 1024;
-    if (R16 <= 64 && a.tc_q_plain) return long_contiguous || 2ll * a.B * a.Hkv >= 3ll * a.tc_ctas;
-    if (R16 <= 64) return paged ? a.max_seq_len > 512 && tokens >= 32 * 1024 : long_contiguous;
-    return R16 <= 80 && a.tc_q_plain && long_contiguous;
+    return R16 <= 32 || (R16 <= 64 && (long long)a.B * a.Hkv >= 3ll * a.tc_ctas);
 }
 
 bool tok_layout(const AttnArgs &a, TokLayout *lay) {
@@ -875,17 +867,15 @@ bool tok_layout(const AttnArgs &a, TokLayout *lay) {
     const int front = (OFF_TAB + tab + 1023) & ~1023;
     const int q = R16 * 256 * (a.tc_q_plain ? 1 : 2), p = STEP * 128 * ((R16 + 63) / 64);
     const int room = SMEM_MAX - 1024 - front - p;
-    const int two = (room - 2 * q) / SLOT, one = (room - q) / SLOT;
+    int slots = (room - 2 * q) / SLOT;
+    if (slots < 4) return false;  // (more than 48 rows in batches with large tables)
     lay->r16 = R16;
-    lay->nq = two >= 4 || two == one ? 2 : 1;
-    int slots = lay->nq == 2 ? two : one;
-    if (slots < 4) return false;
     if (slots > 2 * MAX_SLOTS) slots = 2 * MAX_SLOTS;
     lay->nk = slots / 2;
     lay->nv = slots - lay->nk;
     lay->q_bytes = q;
     lay->off_q = front;
-    lay->off_p = front + lay->nq * q;
+    lay->off_p = front + 2 * q;
     lay->off_k = lay->off_p + p;
     lay->off_v = lay->off_k + lay->nk * SLOT;
     lay->smem = lay->off_v + lay->nv * SLOT + 1024;
@@ -921,7 +911,6 @@ cudaError_t launch_attention_tok(const AttnArgs &a, const CUtensorMap &map_k, co
     case 32: return launch_tok<32>(a, lay, map_k, map_v, st);
     case 48: return launch_tok<48>(a, lay, map_k, map_v, st);
     case 64: return launch_tok<64>(a, lay, map_k, map_v, st);
-    case 80: return launch_tok<80>(a, lay, map_k, map_v, st);
     }
     return cudaErrorInvalidValue;
 }

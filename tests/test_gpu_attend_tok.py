@@ -94,27 +94,34 @@ def _lens(B, longest):
     return [int(x) for x in lens]
 
 
-# the row counts that take this kernel only from some size on: many sequences (64
-# rows plain), long contiguous caches (64 and 80 rows plain)
-@pytest.mark.parametrize("hq,k,layout,B,longest", [
-    (4, 16, wl.LAYOUT_PAGED, 120, 200), (4, 15, wl.LAYOUT_CONTIGUOUS, 115, 129),
-    (4, 16, wl.LAYOUT_CONTIGUOUS, 25, 4200), (5, 16, wl.LAYOUT_CONTIGUOUS, 25, 4200),
+# 33 to 64 rows take this kernel from three (sequence, kv head) pairs per CTA on, 57
+# sequences of 8 kv heads or 228 of 2 on 152 SMs; more rows never do
+@pytest.mark.parametrize("hq,k,layout,B,longest,hkv", [
+    (4, 16, wl.LAYOUT_PAGED, 120, 200, 2), (4, 15, wl.LAYOUT_CONTIGUOUS, 115, 129, 2),
+    (4, 16, wl.LAYOUT_CONTIGUOUS, 25, 4200, 2), (5, 16, wl.LAYOUT_CONTIGUOUS, 25, 4200, 2),
+    (4, 16, wl.LAYOUT_PAGED, 56, 700, 8), (4, 16, wl.LAYOUT_CONTIGUOUS, 57, 700, 8),
+    (4, 16, wl.LAYOUT_PAGED, 300, 1100, 2), (7, 8, wl.LAYOUT_PAGED, 240, 500, 2), (3, 16, wl.LAYOUT_PAGED, 240, 300, 2),
 ])
-def test_plain_queries_from_a_size_on(hq, k, layout, B, longest):
-    w = wl.custom(wl.Shape(256, 2 * hq, 2, 128, 512, k, 2), _lens(B, longest), layout, 730 + k, rows_per_seq=True)
+def test_plain_queries_of_more_rows(hq, k, layout, B, longest, hkv):
+    w = wl.custom(wl.Shape(256, hkv * hq, hkv, 128, 512, k, 2), _lens(B, longest), layout, 730 + k, rows_per_seq=True)
     run = GpuRun(w)
     compare(run.logits(), oracle_logits(w), label=f"plain R={hq * k}")
     run.close()
 
 
-@pytest.mark.parametrize("k,page,B,longest", [(12, 0, 8, 2100), (16, 16, 16, 2100), (16, 0, 25, 4200)])
-def test_exact_queries_from_a_size_on(k, page, B, longest):
+# (1900 sequences: the tables leave too little shared memory for 48 or 64 hi + lo rows)
+@pytest.mark.parametrize("k,page,B,longest,hkv", [
+    (12, 0, 8, 2100, 2), (16, 16, 16, 2100, 2), (16, 0, 25, 4200, 2),
+    (12, 0, 56, 400, 8), (12, 16, 57, 1300, 8), (9, 0, 60, 1300, 8), (12, 64, 1900, 150, 2), (11, 32, 400, 700, 2),
+    (16, 16, 240, 300, 2), (16, 0, 57, 900, 8), (15, 16, 1900, 150, 2),
+])
+def test_exact_queries_of_more_rows(k, page, B, longest, hkv):
     ensure_built()
-    shape = wl.Shape(256, 8, 2, 128, 256, k, 2, page_size=page or 16)
+    shape = wl.Shape(256, 4 * hkv, hkv, 128, 256, k, 2, page_size=page or 16)
     w = wl.custom(shape, _lens(B, longest), wl.LAYOUT_PAGED if page else wl.LAYOUT_CONTIGUOUS, 740 + k)
     rng = np.random.default_rng(k)
-    q = rng.standard_normal((B, k, 8, 128)).astype(np.float32)
-    kn, vn = (rng.standard_normal((B, k, 2, 128)).astype(np.float32) for _ in range(2))
+    q = rng.standard_normal((B, k, 4 * hkv, 128)).astype(np.float32)
+    kn, vn = (rng.standard_normal((B, k, hkv, 128)).astype(np.float32) for _ in range(2))
     ref = so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn)))
     out, _ = _attend(shape, w, q, kn, vn, 2)
     # as above: bf16 new values and scores, 2e-2 in all at 1.5 times these queries
@@ -137,3 +144,20 @@ def test_shares(lens, hq, k):
     for _ in range(2):  # the merge counters are clear again after the first call
         out, _ = _attend(shape, w, q, kn, vn, 2)
         assert np.all(np.abs(out - ref) <= 2e-2 * (1 + np.abs(ref)))
+
+
+@pytest.mark.parametrize("hq,k,layout,B", [
+    (4, 16, wl.LAYOUT_CONTIGUOUS, 16), (5, 16, wl.LAYOUT_CONTIGUOUS, 16), (3, 16, wl.LAYOUT_PAGED, 8),
+    (4, 12, wl.LAYOUT_CONTIGUOUS, 4), (4, 15, wl.LAYOUT_PAGED, 8), (4, 8, wl.LAYOUT_PAGED, 3),
+    (6, 16, wl.LAYOUT_CONTIGUOUS, 16),
+])
+def test_the_length_bound_chooses_nothing(hq, k, layout, B):
+    # max_seq_len is a server's context limit and may be far above every length: the
+    # kernel and its plan, and so the bits, do not depend on it
+    w = wl.custom(wl.Shape(256, 2 * hq, 2, 128, 512, k, 2), _lens(B, 500), layout, 770 + k, rows_per_seq=True)
+    got = []
+    for bound in (500, 33000):
+        run = GpuRun(w, max_seq_len=bound)
+        got.append(run.logits())
+        run.close()
+    assert np.array_equal(got[0], got[1])
