@@ -18,7 +18,21 @@
 //                    then the rare path finds the row maxima and rescales O), row
 //                    sums stay per thread until the segment ends
 //   O^T += V^T P     M = 128 dims (V read in place as the transposed A operand),
-//                    N = query rows, P as bf16 [token][row] in shared memory
+//                    N = query rows, P as bf16 [token][row] in shared memory; on the
+//                    first step of a segment of a short sequence as bf16 hi + lo, two
+//                    MMAs (the lo plane in the free half of P's 128-byte lines up to 32
+//                    rows, else over the step's K, which the scores are done with)
+// Precision: a probability of 1, that of a row's maximum where it sets the running
+// max, is the only one that bf16 holds exactly, and one maximum per 128 tokens leaves
+// more to rounding than the queries-on-M kernel's one per 64.  Against that, the row
+// sums (fp32) are over the probabilities as rounded: an error e of a token's weight
+// then moves the output by e (v - o) instead of e v, never more on average (sum w^2 -
+// 2 sum w^3 + (sum w^2)^2 <= sum w^2); and sequences of up to 256 tokens have the lo
+// plane.  Relative error of the output, 4 rows of 32 heads: 100 tokens 1.45e-3 (queries
+// on M), 1.53e-3 (this kernel with neither), 1.00e-3 (now); 300 tokens 1.64e-3, 1.66e-3,
+// 1.60e-3; 1000 tokens 1.66e-3, 1.67e-3, 1.63e-3; 4000 tokens 1.64e-3 in all.  The sums
+// cost nothing that can be measured, the lo plane 0.3-0.6 % of a call of up to 32 rows
+// that has one and about 0.2 % of others.
 // An MMA costs the padded row count instead of 128 columns (40 cycles at 32 rows,
 // shared-memory bandwidth of the token operand), and a step of 128 tokens takes
 // 1.2-1.4 us while all SMs stream: HBM-bound (7 TB/s between a segment's first and
@@ -55,6 +69,7 @@ constexpr int OFF_ROW = 512;               // per-row tables and reductions
 constexpr int ROW_WORDS = 11 * 128;
 constexpr int OFF_CUT = OFF_ROW + ROW_WORDS * 4;
 constexpr int OFF_TAB = OFF_CUT + (MAX_GRP + 4) * 4;  // prefix [B + 1], (sid, len) [B]
+constexpr int LO_TILES = 4;                // P has a lo plane in sequences of up to 256 tokens
 constexpr int THREADS = 512;
 constexpr int PROD_WARP = 8, Q_WARP = 12, MMA_W = 15;
 constexpr int SOFT_THREADS = 256, KV_THREADS = 64, Q_THREADS = 96;
@@ -167,6 +182,7 @@ struct Walk {
     }
     __device__ __forceinline__ bool done() const { return n == 0; }
     __device__ __forceinline__ int tiles() const { return min(2, sg.n - 2 * i); }  // of this step
+    __device__ __forceinline__ bool lo() const { return i == 0 && sg.nt <= LO_TILES; }
     __device__ __forceinline__ void next() {
         if (++i == n) seg();
     }
@@ -241,6 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr uint32_t O_COL = 2 * S_COLS;
     constexpr uint32_t TMEM_COLS = NR <= 32 ? 128 : 256;
     static_assert(NR % 16 == 0 && NR <= 64, "query rows");
+    constexpr bool LO_IN_LINE = NR <= 32;        // P's lo plane in P's lines, else in the K slot
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     TokBars *bars = (TokBars *)(smem + OFF_BAR);
@@ -491,6 +508,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint64_t dq0 = sw128_kmajor_desc(smem + lay.off_q);
         const uint64_t dv0 = sw128_mnmajor_desc2(smem + lay.off_v, HALF_STRIDE, GROUP_STRIDE);
         const uint64_t dp0 = sw128_mnmajor_desc2(smem + lay.off_p, STEP * 128, 1024);
+        const uint64_t dl0 = sw128_mnmajor_desc2(smem + lay.off_k, STEP * 128, 1024);
         const uint32_t q_step = (uint32_t)lay.q_bytes >> 4;
         const bool q_lo = !a.tc_q_plain;
         Walk ws(prefix, B, x0, x1);
@@ -516,7 +534,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     mma_bf16(d, ak, bq, idesc_s, kk > 0 ? 1u : 0u);
                     if (q_lo) mma_bf16(d, ak, bq + (uint64_t)(NR * 256 >> 4), idesc_s, 1u);
                 }
-                mma_commit(&bars->k_empty[rk.slot]);
+                if (LO_IN_LINE || !ws.lo()) mma_commit(&bars->k_empty[rk.slot]);
                 mma_commit(&bars->s_full[sbuf]);
                 if (ws.i == ws.n - 1) mma_commit(&bars->q_empty[rq.slot]);
             }
@@ -527,6 +545,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         };
         issue_s();
         issue_s();
+        Ring rp(lay.nk);  // the step's K slot
         uint32_t ph = 0;
 #pragma unroll 1
         for (Walk w(prefix, B, x0, x1); ok && !w.done(); w.next(), ph ^= 1) {
@@ -542,10 +561,20 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (kk < TT / 16 || two)
                         mma_bf16(tmem + O_COL, dv + (uint64_t)(kk * (2 * GROUP_STRIDE >> 4)),
                                  dp0 + (uint64_t)(kk * (2048 >> 4)), idesc_o, (w.i > 0 || kk > 0) ? 1u : 0u);
+                if (w.lo()) {
+                    const uint64_t dl = LO_IN_LINE ? dp0 + (64 >> 4) : dl0 + (uint32_t)(rp.slot * (SLOT >> 4));
+#pragma unroll
+                    for (int kk = 0; kk < STEP / 16; ++kk)
+                        if (kk < TT / 16 || two)
+                            mma_bf16(tmem + O_COL, dv + (uint64_t)(kk * (2 * GROUP_STRIDE >> 4)),
+                                     dl + (uint64_t)(kk * (2048 >> 4)), idesc_o, 1u);
+                    if (!LO_IN_LINE) mma_commit(&bars->k_empty[rp.slot]);
+                }
                 mma_commit(&bars->v_empty[rv.slot]);
                 mma_commit(&bars->pv_done);
             }
             rv.next();
+            rp.next();
             issue_s();
         }
         if (lead) mma_commit(&bars->fin);  // completes when every MMA is done
@@ -688,14 +717,37 @@ __global__ void __launch_bounds__(THREADS, 1)
                             p1 = fast_exp2(p1);
                             p2 = fast_exp2(p2);
                             p3 = fast_exp2(p3);
-                            add2(l[cj], l[cj + 1], l[cj], l[cj + 1], p0, p1);
-                            add2(l[cj + 2], l[cj + 3], l[cj + 2], l[cj + 3], p2, p3);
-                            pk[2 * h] = pack_bf16(p0, p1);
-                            pk[2 * h + 1] = pack_bf16(p2, p3);
+                            const uint32_t u0 = pack_bf16(p0, p1), u1 = pack_bf16(p2, p3);
+                            add2(l[cj], l[cj + 1], l[cj], l[cj + 1], __uint_as_float(u0 << 16),
+                                 __uint_as_float(u0 & 0xffff0000u));
+                            add2(l[cj + 2], l[cj + 3], l[cj + 2], l[cj + 3], __uint_as_float(u1 << 16),
+                                 __uint_as_float(u1 & 0xffff0000u));
+                            pk[2 * h] = u0;
+                            pk[2 * h + 1] = u1;
                         }
-                        const int c16 = (cb + c * W + j8) >> 3;  // 16-byte chunk: 64 rows per 128-byte line
-                        st_shared_v4(prow + (c16 >> 3) * (STEP * 128) + (((c16 & 7) ^ (tok & 7)) << 4), pk[0], pk[1],
-                                     pk[2], pk[3]);
+                        const int c16 = (cb + c * W + j8) >> 3;  // 16-byte chunk of the line
+                        st_shared_v4(prow + ((c16 ^ (tok & 7)) << 4), pk[0], pk[1], pk[2], pk[3]);
+                    }
+                }
+                if (i == 0 && sg.nt <= LO_TILES) {  // uniform
+                    // (every step takes the next of the nk K slots)
+                    uint8_t *lrow = LO_IN_LINE ? prow : prow + (lay.off_k - lay.off_p) + n % lay.nk * SLOT;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+                        for (int j8 = 0; j8 < W; j8 += 8) {
+                            const float *nm = nm_s + cb + c * W + j8;
+                            float e[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const float p = fast_exp2(sv[c][j8 + j] + nm[j]);
+                                e[j] = p - __bfloat162float(__float2bfloat16_rn(p));
+                                l[c * W + j8 + j] += e[j];
+                            }
+                            const int c16 = ((cb + c * W + j8) >> 3) + (LO_IN_LINE ? 4 : 0);
+                            st_shared_v4(lrow + ((c16 ^ (tok & 7)) << 4), pack_bf16(e[0], e[1]), pack_bf16(e[2], e[3]),
+                                         pack_bf16(e[4], e[5]), pack_bf16(e[6], e[7]));
+                        }
                     }
                 }
                 fence_proxy_async();
@@ -865,7 +917,7 @@ bool tok_layout(const AttnArgs &a, TokLayout *lay) {
     if (!tok_wins(a, R16)) return false;
     const int tab = ((a.B + 2) & ~1) * 4 + a.B * 8;
     const int front = (OFF_TAB + tab + 1023) & ~1023;
-    const int q = R16 * 256 * (a.tc_q_plain ? 1 : 2), p = STEP * 128 * ((R16 + 63) / 64);
+    const int q = R16 * 256 * (a.tc_q_plain ? 1 : 2), p = STEP * 128;
     const int room = SMEM_MAX - 1024 - front - p;
     int slots = (room - 2 * q) / SLOT;
     if (slots < 4) return false;  // (more than 48 rows in batches with large tables)
