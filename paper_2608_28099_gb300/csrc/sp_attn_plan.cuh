@@ -74,15 +74,20 @@ __device__ __forceinline__ Seg seg_at(const int *prefix, int B, int x, int x_end
 //     it (a short piece of a sequence would pay a whole segment);
 //   whole: a cut within half a virtual share of a sequence start moves onto it, so
 //     that sequences shorter than a share are never split.
-// and the one whose largest share (tiles + c per segment) is smaller is taken:
-// near where sequences are longer or many more than the shares, whole where they
-// are about as many.  The cuts never decrease; two may meet at a sequence start,
-// and the share between them is then empty (four sequences of 15 tiles in eight
-// shares).
+// and the one whose largest share is smaller is taken, counting its tiles, c per
+// segment and MERGE_COST for each of its ends inside a sequence (a partial to write
+// and to merge; nothing where a kernel of its own merges): near where sequences are
+// longer or many more than the shares, whole where they are about as many.  The cuts
+// never decrease; two may meet at a sequence start, and the share between them is
+// then empty (four sequences of 15 tiles in eight shares).
 // Attention step (8 kv heads, 152 SMs) with near alone -> the choice, paged, 96 query
 // rows: 16 x 500 tokens 44.5 -> 22.3 us, 16 x 1000 47.4 -> 26.8; 16 rows, 16 x 1000:
-// 20.2 -> 17.5.
+// 20.2 -> 17.5.  MERGE_COST 0 and 4, 8 sequences of 60 to 203 tokens, 16 / 32 / 96
+// rows: 23.6 / 29.7 / 42.0 and 19.5 / 21.5 / 29.7 us.  Of 2160 batches (6 to 32
+// sequences of 36 to 6800 tokens, 16 to 128 rows) the choice took on average 4.4 % more
+// than the better plan without it, 0.7 % with 4 (2: 1.4, 8: 0.9).
 constexpr int SNAP = 4;
+constexpr int MERGE_COST = 4;
 constexpr int PLAN_THREADS = 128;
 constexpr int PLAN_BAR = 15;  // named barrier of the planning warps
 
@@ -126,16 +131,19 @@ __device__ __forceinline__ void share_cut(const int *prefix, int B, int T, int n
     *whole = e0 <= e1 && e0 <= half ? Cut{p0, lo} : e1 <= half ? Cut{p1, lo + 1} : Cut{x, lo};
 }
 
-// Tiles and segments of the share [a, b).
-__device__ __forceinline__ int share_cost(const int *prefix, Cut a, Cut b, int c) {
+// Tiles, segments and ends inside a sequence (m each) of the share [a, b).
+__device__ __forceinline__ int share_cost(const int *prefix, Cut a, Cut b, int c, int m) {
     if (b.x <= a.x) return 0;
-    return b.x - a.x + c * (b.s - (b.x == prefix[b.s]) - a.s + 1);
+    const int cut_a = a.x != prefix[a.s], cut_b = b.x != prefix[b.s];
+    return b.x - a.x + c * (b.s + cut_b - a.s) + m * (cut_a + cut_b);
 }
 
 // cuts[0 .. n] by the first PLAN_THREADS threads; worst: two ints per warp.  A
 // warp's lane 31 holds the next warp's first cut.  The caller synchronises.
-__device__ __forceinline__ void build_cuts(const int *prefix, int B, int T, int n, int c, int *cuts, int *worst) {
+__device__ __forceinline__ void build_cuts(const AttnArgs &args, const int *prefix, int T, int n, int *cuts,
+                                           int *worst) {
     constexpr int PER = 31 * (PLAN_THREADS / 32);
+    const int B = args.B, c = args.tc_seg_cost, m = args.tc_merge_kernel ? 0 : MERGE_COST;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Cut near, whole;
     int m0 = 0, m1 = 0;
@@ -149,8 +157,8 @@ __device__ __forceinline__ void build_cuts(const int *prefix, int B, int T, int 
         b1.x = __shfl_down_sync(0xffffffffu, whole.x, 1);
         b1.s = __shfl_down_sync(0xffffffffu, whole.s, 1);
         if (lane < 31 && j < n) {
-            m0 = max(m0, share_cost(prefix, near, b0, c));
-            m1 = max(m1, share_cost(prefix, whole, b1, c));
+            m0 = max(m0, share_cost(prefix, near, b0, c, m));
+            m1 = max(m1, share_cost(prefix, whole, b1, c, m));
         }
     }
     m0 = __reduce_max_sync(0xffffffffu, m0);

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         return;
     }
     int *cuts = (int *)(smem + OFF_CUTS);
-    if (threadIdx.x < PLAN_THREADS) build_cuts(prefix, B, T, n_grp, a.tc_seg_cost, cuts, bars->wsum);
+    if (threadIdx.x < PLAN_THREADS) build_cuts(a, prefix, T, n_grp, cuts, bars->wsum);
     __syncthreads();
     const int x0 = cuts[grp], x1 = cuts[grp + 1];
 
@@ -760,7 +760,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) attn_tc_merge_kernel(AttnArgs a)
     build_prefix<PLAN_THREADS>(a, prefix, nullptr, scratch, nullptr);
     const int T = prefix[B];
     const int n_grp = share_count(a.tc_ctas / Hkv, T, B, a.tc_min_tiles);
-    build_cuts(prefix, B, T, n_grp, a.tc_seg_cost, cuts, scratch);
+    build_cuts(a, prefix, T, n_grp, cuts, scratch);
     __syncthreads();
     const int j0 = group_of(cuts, n_grp, prefix[b]);
     const int j1 = group_of(cuts, n_grp, prefix[b + 1] - 1);

@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         return;
     }
     if (threadIdx.x < PLAN_THREADS)  // (set-up is shared out over the warps)
-        build_cuts(prefix, B, T, n_grp, a.tc_seg_cost, cuts, bars->wsum);
+        build_cuts(a, prefix, T, n_grp, cuts, bars->wsum);
     if (threadIdx.x >= 128 && threadIdx.x < 256) {
         const int rr = threadIdx.x - 128;
         const int rk = rr % k;

@@ -211,3 +211,30 @@ def test_error_is_no_larger_than_that_of_the_kernel_with_queries_on_m(L, k, hq, 
     out, _ = _attend(shape, w, q, kn, vn, 2, split=0)
     err, want = np.linalg.norm(out - ref), np.linalg.norm(other - ref)
     assert err <= 1.02 * want, (err / np.linalg.norm(ref), want / np.linalg.norm(ref))
+
+
+@pytest.mark.parametrize("k,lens", [
+    (4, [160, 80, 143, 98, 105, 91]), (8, [187, 156, 154, 133, 117, 45, 116, 140]),
+    (8, [54, 144, 133, 67, 82, 185, 72, 163, 117, 200, 175, 141, 131, 57, 108, 77]),
+    (16, [105, 99, 62, 113, 185, 91, 59, 72, 50, 68, 48, 199]), (24, [60, 154, 125, 202, 203, 133, 174, 91]),
+    (32, [184, 145, 91, 157, 195, 56, 81, 43, 126, 126]),
+])
+def test_short_sequences_stay_whole(k, lens):
+    # a sequence that no share cut: the same bits as alone, where (up to 256 tokens
+    # with the new ones) it is one share
+    ensure_built()
+    shape = wl.Shape(256, 32, 8, 128, 256, k, 2)
+    w = wl.custom(shape, lens, wl.LAYOUT_CONTIGUOUS, 780 + k)
+    rng = np.random.default_rng(k)
+    B = len(lens)
+    q = rng.standard_normal((B, k, 32, 128)).astype(np.float32)
+    kn, vn = (rng.standard_normal((B, k, 8, 128)).astype(np.float32) for _ in range(2))
+    out, _ = _attend(shape, w, q, kn, vn, 2, split=0)
+    for b in range(B):
+        o, n = int(w.cache.offsets[b]), lens[b]
+        c = w.cache
+        alone = wl.KVCache(c.layout, c.dtype, np.array([n], np.int32), c.k_flat[o:o + n], c.v_flat[o:o + n],
+                           np.array([0], np.int64))
+        one = wl.Workload(w.spec, w.weights, alone, np.array([0], np.int32), None)
+        got, _ = _attend(shape, one, q[b:b + 1], kn[b:b + 1], vn[b:b + 1], 2, split=0)
+        assert np.array_equal(got[0], out[b]), b
