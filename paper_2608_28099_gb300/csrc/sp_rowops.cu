@@ -512,9 +512,13 @@ readout_kernel(PartIn y, const float *__restrict__ h1, const float *__restrict__
         __threadfence();  // the warp's partials are visible before the block is counted
         is_last = atomicAdd(counters + b, 1) == (int)gridDim.x - 1;
         if (is_last) counters[b] = 0;
-        __threadfence();  // the other blocks' partials are read after their count
     }
     if (!__shfl_sync(0xffffffffu, is_last, 0)) return;
+    // the other blocks' partials are read after their count: a fence in every lane
+    // that reads (a shuffle orders no memory), behind the barrier that lane 0's
+    // atomic comes before
+    __syncwarp();
+    __threadfence();
     const int n_chunks = gridDim.x;
     float inv = 1.f;  // 1 / rms of the pooled row (LM-head readout)
     if (g_final) {

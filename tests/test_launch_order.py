@@ -80,3 +80,12 @@ def test_a_first_kernel_reads_the_callers_data_after_its_wait(name):
     before = KERNELS[name]
     before = before[:before.index("pdl_wait()")]
     assert not re.search(r"resolve_seq|load_tile\(|load4\(|load8\(|\bx\[|\bX\[|\bW\[|xr\b", before)
+
+
+def test_readout_lanes_fence_between_the_count_and_the_other_blocks_partials():
+    # one lane counts the block; every lane of the last block reads partials that
+    # other blocks wrote, so each needs its own fence after it learns the verdict
+    body = KERNELS["readout_kernel"]
+    after = body[body.index("__shfl_sync(0xffffffffu, is_last"):]
+    before_reads = after[:after.index("__ldcg(")]
+    assert "__syncwarp()" in before_reads and "__threadfence()" in before_reads
