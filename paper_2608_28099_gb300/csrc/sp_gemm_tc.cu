@@ -635,6 +635,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 2)  /*
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort && g.status) atomicOr(g.status, SP_DEV_TIMEOUT);
+    // rank 0's last commit arrives on both CTAs' barriers: each waits until it has
+    // landed in its own shared memory (rank 0 did above)
+    if (threadIdx.x == 0 && rank != 0) mbar_wait_drain(fin, 0, g.wait_ns);
+    __syncwarp();
     cluster_sync();  // no signal or MMA of the other CTA may still target this one
     if (warp == PAIR_TMEM) tmem_dealloc_pair(tmem, Cfg::TMEM_COLS);
 }

@@ -89,3 +89,11 @@ def test_readout_lanes_fence_between_the_count_and_the_other_blocks_partials():
     after = body[body.index("__shfl_sync(0xffffffffu, is_last"):]
     before_reads = after[:after.index("__ldcg(")]
     assert "__syncwarp()" in before_reads and "__threadfence()" in before_reads
+
+
+def test_both_ctas_of_a_pair_wait_for_what_arrives_on_their_barriers():
+    # a commit of the pair arrives on the barrier of both CTAs; one that left before
+    # the arrival landed would have it written into the next block's shared memory
+    body = KERNELS["gemm_pair_kernel"]
+    end = body[body.rindex("__syncthreads()"):]
+    assert re.search(r"rank\s*!=\s*0\s*\)\s*mbar_wait_drain\(fin\b", end[:end.index("cluster_sync()")])
