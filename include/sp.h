@@ -265,8 +265,8 @@ enum {
                                  always, 4 = plain bf16 except Q/K/V            */
     SP_OPT_DEBUG_STALL = 8,   /* test of the failure path: 1 = in the next
                                  sp_classify only, the first CTA of the output
-                                 projection (when it runs on the one-CTA-per-tile
-                                 schedule) never loads its first k-block, so its
+                                 projection (unless it runs on the persistent
+                                 stream-K schedule) never loads its first k-block, so its
                                  tensor-core wait runs out; that launch's waits
                                  give up after 1 ms, the kernel drains its copies,
                                  frees TMEM and returns, and sp_check_status

@@ -177,8 +177,7 @@ struct GemmPlanner {
                   const RopeEpi *rope = nullptr) const {
         cudaError_t e;
         if (use_tc(w, x, path)) {
-            TcPlan p = tc_plan(M, w.N, w.K, n_sm, y_capacity, lo, sched);
-            if (inject_stall) p.pair = false;  // the failure-path test is the tile kernel's
+            const TcPlan p = tc_plan(M, w.N, w.K, n_sm, y_capacity, lo, sched);
             const int bi = bn_index(p.box_rows(lo));
             e = launch_gemm_tc(w.map, x.hi[bi], x.lo[bi], p, M, w.N, w.K, y, status, st, w.blocked, lo,
                                inject_stall, glu, rope);

@@ -493,16 +493,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 2)  /*
         };
         int m0, tile, kb0, nkb, split, gi = 0, pre = 0;
         bool ok = true;
+        const bool skip0 = g.inject_stall && blockIdx.x == 0;  // rank 0's first k-block
         if (cl < n_items) {
             item(cl, m0, tile, kb0, nkb, split);
             pre = min(nkb, Cfg::STAGES);
-            for (int i = 0; i < pre; ++i) load_w(i, tile, kb0 + i);
+            for (int i = skip0 ? 1 : 0; i < pre; ++i) load_w(i, tile, kb0 + i);
         }
         pdl_wait();
         for (int it = cl; ok && it < n_items; it += n_cl) {
             item(it, m0, tile, kb0, nkb, split);
             for (int i = 0; i < nkb; ++i, ++gi) {
                 const int s = gi % Cfg::STAGES;
+                if (skip0 && gi == 0) continue;
                 if (gi >= pre) {
                     if (!mbar_wait(&empty[s], ((gi / Cfg::STAGES) & 1) ^ 1, abort, g.wait_ns)) {
                         ok = false;

@@ -38,3 +38,22 @@ def test_pair_epilogues(B, k, precision):
                   options={sp.SP_OPT_ACT_PRECISION: precision})
     compare(run_.logits(), oracle_logits(w), label=f"pair B={B} k={k}")
     run_.close()
+
+
+def test_wait_timeout_is_reported_and_the_handle_recovers():
+    # the failure path across the two CTAs: rank 0 of the first pair never loads its
+    # first k-block, the MMA and every wait of both CTAs behind it give up after 1 ms,
+    # both drain, free TMEM and return; nothing faults
+    sh = wl.Shape(256, 8, 2, 128, 512, 4, 3)
+    run_ = GpuRun(w := wl.custom(sh, [20, 300, 64, 5] * 6, wl.LAYOUT_PAGED, 621, rows_per_seq=True))
+    torch, h = run_.torch, run_.model.handle
+    plan = sp.sp_debug_gemm_plan(96, 256, 1024, 152, 1)  # output projection: 128-row hi + lo tiles, eight items
+    assert (plan["rows_per_tile"], plan["n_tiles"], plan["persistent"]) == (128, 2, 0)
+    out = torch.empty((24, 3), device="cuda")
+    for _ in range(2):
+        sp.sp_set_option(h, sp.SP_OPT_DEBUG_STALL, 1)
+        sp.sp_classify(h, torch.cuda.current_stream(), 24, run_.ids, run_.cache.seq_lens, run_.cache.desc,
+                       run_.rows, out)
+        assert sp.sp_check_status(h) & sp.SP_DEV_TIMEOUT
+        compare(run_.logits(), oracle_logits(w), label="after timeout")
+    run_.close()
