@@ -26,13 +26,14 @@
 // max, is the only one that bf16 holds exactly, and one maximum per 128 tokens leaves
 // more to rounding than the queries-on-M kernel's one per 64.  Against that, the row
 // sums (fp32) are over the probabilities as rounded: an error e of a token's weight
-// then moves the output by e (v - o) instead of e v, never more on average (sum w^2 -
-// 2 sum w^3 + (sum w^2)^2 <= sum w^2); and sequences of up to 256 tokens have the lo
-// plane.  Relative error of the output, 4 rows of 32 heads: 100 tokens 1.45e-3 (queries
-// on M), 1.53e-3 (this kernel with neither), 1.00e-3 (now); 300 tokens 1.64e-3, 1.66e-3,
-// 1.60e-3; 1000 tokens 1.66e-3, 1.67e-3, 1.63e-3; 4000 tokens 1.64e-3 in all.  The sums
-// cost nothing that can be measured, the lo plane 0.3-0.6 % of a call of up to 32 rows
-// that has one and about 0.2 % of others.
+// then moves the output by e (v - o) instead of e v, never more on average over values of
+// one distribution (sum w^2 - 2 sum w^3 + (sum w^2)^2 <= sum w^2); and sequences of up to
+// 512 tokens have the lo plane (256 from 33 rows on, where holding the K slot costs
+// 2-3 % of a call beyond).  Relative error of the output, 4 rows of 32 heads: 100 tokens
+// 1.45e-3 (queries on M), 1.53e-3 (this kernel with neither), 1.00e-3 (now); 300 tokens
+// 1.64e-3, 1.66e-3, 1.41e-3; 1000 tokens 1.66e-3, 1.67e-3, 1.63e-3; 4000 tokens 1.64e-3 in
+// all.  The sums cost nothing that can be measured, the lo plane 0.3-0.6 % of a call of
+// up to 32 rows that has one and about 0.2 % of others.
 // An MMA costs the padded row count instead of 128 columns (40 cycles at 32 rows,
 // shared-memory bandwidth of the token operand), and a step of 128 tokens takes
 // 1.2-1.4 us while all SMs stream: HBM-bound (7 TB/s between a segment's first and
@@ -69,7 +70,6 @@ constexpr int OFF_ROW = 512;               // per-row tables and reductions
 constexpr int ROW_WORDS = 11 * 128;
 constexpr int OFF_CUT = OFF_ROW + ROW_WORDS * 4;
 constexpr int OFF_TAB = OFF_CUT + (MAX_GRP + 4) * 4;  // prefix [B + 1], (sid, len) [B]
-constexpr int LO_TILES = 4;                // P has a lo plane in sequences of up to 256 tokens
 constexpr int THREADS = 512;
 constexpr int PROD_WARP = 8, Q_WARP = 12, MMA_W = 15;
 constexpr int SOFT_THREADS = 256, KV_THREADS = 64, Q_THREADS = 96;
@@ -182,7 +182,6 @@ struct Walk {
     }
     __device__ __forceinline__ bool done() const { return n == 0; }
     __device__ __forceinline__ int tiles() const { return min(2, sg.n - 2 * i); }  // of this step
-    __device__ __forceinline__ bool lo() const { return i == 0 && sg.nt <= LO_TILES; }
     __device__ __forceinline__ void next() {
         if (++i == n) seg();
     }
@@ -258,6 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr uint32_t TMEM_COLS = NR <= 32 ? 128 : 256;
     static_assert(NR % 16 == 0 && NR <= 64, "query rows");
     constexpr bool LO_IN_LINE = NR <= 32;        // P's lo plane in P's lines, else in the K slot
+    constexpr int LO_TILES = LO_IN_LINE ? 8 : 4; // sequences (tiles) that have one: 512 or 256 tokens
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     TokBars *bars = (TokBars *)(smem + OFF_BAR);
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     mma_bf16(d, ak, bq, idesc_s, kk > 0 ? 1u : 0u);
                     if (q_lo) mma_bf16(d, ak, bq + (uint64_t)(NR * 256 >> 4), idesc_s, 1u);
                 }
-                if (LO_IN_LINE || !ws.lo()) mma_commit(&bars->k_empty[rk.slot]);
+                if (LO_IN_LINE || ws.i > 0 || ws.sg.nt > LO_TILES) mma_commit(&bars->k_empty[rk.slot]);
                 mma_commit(&bars->s_full[sbuf]);
                 if (ws.i == ws.n - 1) mma_commit(&bars->q_empty[rq.slot]);
             }
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (kk < TT / 16 || two)
                         mma_bf16(tmem + O_COL, dv + (uint64_t)(kk * (2 * GROUP_STRIDE >> 4)),
                                  dp0 + (uint64_t)(kk * (2048 >> 4)), idesc_o, (w.i > 0 || kk > 0) ? 1u : 0u);
-                if (w.lo()) {
+                if (w.i == 0 && w.sg.nt <= LO_TILES) {
                     const uint64_t dl = LO_IN_LINE ? dp0 + (64 >> 4) : dl0 + (uint32_t)(rp.slot * (SLOT >> 4));
 #pragma unroll
                     for (int kk = 0; kk < STEP / 16; ++kk)
