@@ -21,8 +21,8 @@ constexpr int MAX_GRP = 256;                   // groups (cuts table in smem)
 constexpr float RESCALE_LOG2 = 8.f;            // tolerate p <= 2^8 before rescaling O
 constexpr int kStagedSegs = 4;                 // most partials merged through the idle ring
 
-// byte offset of 16-byte chunk c16 (0..15, 8 dims each) of token row `row`
-// (0..63) in a K or V tile
+// byte offset of 16-byte chunk c16 (0..15, 8 dims each) of token row `row` in a K or
+// V slot (one tile of 64 rows, or a step of two: 0..127)
 __device__ __forceinline__ uint32_t kv_off(int row, int c16) {
     return (uint32_t)((row >> 3) * GROUP_STRIDE + (c16 >> 3) * HALF_STRIDE + (row & 7) * 128 +
                       (((c16 & 7) ^ (row & 7)) << 4));
@@ -79,7 +79,7 @@ __device__ __forceinline__ Seg seg_at(const int *prefix, int B, int x, int x_end
 // and to merge; nothing where a kernel of its own merges): near where sequences are
 // longer or many more than the shares, whole where they are about as many.  The cuts
 // never decrease; two may meet at a sequence start, and the share between them is
-// then empty (four sequences of 15 tiles in eight shares).
+// then empty (every other one for four sequences of 15 tiles in eight shares).
 // Attention step (8 kv heads, 152 SMs) with near alone -> the choice, paged, 96 query
 // rows: 16 x 500 tokens 44.5 -> 22.3 us, 16 x 1000 47.4 -> 26.8; 16 rows, 16 x 1000:
 // 20.2 -> 17.5.  MERGE_COST 0 and 4, 8 sequences of 60 to 203 tokens, 16 / 32 / 96
@@ -244,8 +244,8 @@ __device__ __forceinline__ void build_prefix(const AttnArgs &a, int *prefix, int
 // CTA: every partial of the pair lands in the idle K/V ring in one
 // round of cp.async copies (O of segment e as [e][row][dh], then (max,
 // sum) as [e][row]), then thread (row, c) combines 16-byte units c, c + 8,
-// c + 16, c + 24 of its row in segment order, in the arithmetic of the
-// register merge above, so the bits do not depend on which path ran.
+// c + 16, c + 24 of its row in segment order, in the arithmetic of the attention
+// kernels' own merge through registers, so the bits do not depend on which path ran.
 // Shared-memory reads are conflict-free and eight lanes store 64
 // contiguous bytes per plane.  Loads through registers would need a
 // dependent round trip per two segments, each waiting behind the other

@@ -49,9 +49,11 @@ def test_rows_lengths_and_splits(hq, hkv, k, page, split):
 
 
 @pytest.mark.parametrize("hq,k", [(4, 4), (4, 16), (8, 16)])
-def test_empty_share(hq, k):
-    # four sequences of 15 tiles: the first cut between CTA shares snaps to 0, so
-    # the first group of CTAs has nothing to do
+@pytest.mark.parametrize("split", [0, 512])
+def test_empty_share(hq, k, split):
+    # four sequences of 15 tiles.  In shares of eight tiles and more the cuts are 0, 0,
+    # 15, 15, 30, ...: every other group of CTAs, the first one too, has nothing to do.
+    # In the default ones (four and more) two cuts meet in the middle, at 30.
     ensure_built()
     shape = wl.Shape(256, 2 * hq, 2, 128, 256, k, 2)
     w = wl.custom(shape, [900 - 4 * (k > 4)] * 4, wl.LAYOUT_PAGED, 710 + k)
@@ -60,7 +62,7 @@ def test_empty_share(hq, k):
     kn, vn = (rng.standard_normal((4, k, 2, 128)).astype(np.float32) for _ in range(2))
     ref = so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn)))
     for _ in range(2):  # the merge counters are clear again after the first call
-        out, _ = _attend(shape, w, q, kn, vn, 2, split=0)
+        out, _ = _attend(shape, w, q, kn, vn, 2, split=split)
         np.testing.assert_allclose(out, ref, rtol=1e-2, atol=1e-2)
 
 

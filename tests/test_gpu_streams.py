@@ -95,3 +95,87 @@ def test_attend_reads_a_cache_that_the_call_before_it_writes(lens):
     for i, o in enumerate(outs):
         # values off by up to 4e-5 of the largest (hi + lo inputs, K = 1024), the rest fp32
         np.testing.assert_allclose(o.cpu().numpy(), refs[i % 3], rtol=1e-3, atol=1e-3)
+
+
+@pytest.mark.parametrize("recursive", [0, 1])
+def test_hidden_states(recursive):
+    sh = wl.Shape(256, 8, 2, 128, 512, 4, 3)
+    w = wl.with_fusion(wl.custom(sh, [120, 700, 3], wl.LAYOUT_PAGED, 950))
+    run = GpuRun(w, options={sp.SP_OPT_RECURSIVE: recursive})
+    torch, B = run.torch, 3
+    rng = np.random.default_rng(3)
+    states = [wl.f32_to_bf16_bits(rng.standard_normal((B, 256)).astype(np.float32)) for _ in range(3)]
+    layer = so.Layer(w.shape, w.weights)
+    ref = [so.classify_recursive(layer, w.cache, w.seq_ids, s) if recursive
+           else so.classify(layer, w.cache, w.seq_ids, hidden=s) for s in states]
+    dev = [rows_tensor(torch, s) for s in states]
+    outs = [torch.empty((B, 3), device="cuda") for _ in range(12)]
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    for i, o in enumerate(outs):
+        sp.sp_classify_hidden(run.model.handle, st, B, run.ids, run.cache.seq_lens, run.cache.desc, dev[i % 3], o)
+    st.synchronize()
+    for i, o in enumerate(outs):
+        compare(o.double().cpu().numpy(), ref[i % 3], label=f"call {i}")
+        assert torch.equal(o, outs[i % 3])
+    run.close()
+
+
+@pytest.mark.parametrize("M,N,K,path", [(7, 256, 192, 0), (300, 512, 256, 2), (40, 384, 128, 1)])
+def test_project(M, N, K, path):
+    ensure_built()
+    torch = torch_dev()
+    rng = np.random.default_rng(M)
+    # the weights are an argument, too: another matrix in every turn, written in front
+    # of the call on the same stream
+    xs, ws = ([rng.standard_normal((r, K)).astype(np.float32) for _ in range(3)] for r in (M, N))
+    bits = [wl.f32_to_bf16_bits(0.05 * w) for w in ws]
+    ref = [x.astype(np.float64) @ wl.bf16_bits_to_f32(b).astype(np.float64).T for x, b in zip(xs, bits)]
+    x_d = [torch.from_numpy(x).cuda() for x in xs]
+    w_d = [torch.from_numpy(b.view(np.int16)).cuda() for b in bits]
+    x, w = torch.empty_like(x_d[0]), torch.empty_like(w_d[0])
+    n = max(256, sp.sp_project_workspace_bytes(M, N, K))
+    scratch = torch.empty(n, dtype=torch.uint8, device="cuda")
+    outs = [torch.empty((M, N), device="cuda") for _ in range(24)]
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        for i, o in enumerate(outs):
+            x.copy_(x_d[i % 3])
+            w.copy_(w_d[i % 3])
+            sp.sp_project(st, M, N, K, x, w, o, path, scratch, n)
+    st.synchronize()
+    for i, o in enumerate(outs):
+        # hi + lo activations and fp32 sums (the bound of the projection tests)
+        assert np.max(np.abs(o.double().cpu().numpy() - ref[i % 3])) <= 2e-5 * np.max(np.abs(ref[i % 3]))
+
+
+@pytest.mark.parametrize("lens", [[250, 30], [900, 0, 1500, 64], [100] * 40])
+@pytest.mark.parametrize("k", [4, 24])
+def test_attend_on_tensor_cores(lens, k):
+    ensure_built()
+    torch = torch_dev()
+    shape, B = wl.Shape(256, 8, 2, 128, 256, k, 2), len(lens)
+    w = wl.custom(shape, lens, wl.LAYOUT_PAGED, 960)
+    rng = np.random.default_rng(k)
+    qs = [rng.standard_normal((B, k, 8, 128)).astype(np.float32) for _ in range(3)]
+    kn, vn = (rng.standard_normal((B, k, 2, 128)).astype(np.float32) for _ in range(2))
+    ref = [so.attention_step(shape, w.cache, w.seq_ids, *(t.astype(np.float64) for t in (q, kn, vn))) for q in qs]
+    cache = sp.DeviceCache(w.cache)
+    dims = sp.sp_attn_dims(8, 2, 128, k, sp.SP_BF16, max(lens), 0, 2)
+    ws = torch.empty(sp.sp_attend_workspace_bytes(dims, B), dtype=torch.uint8, device="cuda")
+    q_d = [torch.from_numpy(q).cuda() for q in qs]
+    kn_d, vn_d = torch.from_numpy(kn).cuda(), torch.from_numpy(vn).cuda()
+    q = torch.empty_like(q_d[0])
+    outs = [torch.empty(q.shape, device="cuda") for _ in range(24)]
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        for i, o in enumerate(outs):
+            q.copy_(q_d[i % 3])
+            sp.sp_attend(st, dims, B, None, cache.seq_lens, cache.desc, q, kn_d, vn_d, o, sp.SP_F32, ws, ws.numel())
+    st.synchronize()
+    for i, o in enumerate(outs):
+        # bf16 new rows and probabilities (as in the other tests of this step)
+        assert np.all(np.abs(o.cpu().numpy() - ref[i % 3]) <= 2e-2 * (1 + np.abs(ref[i % 3])))
+        assert torch.equal(o, outs[i % 3])
