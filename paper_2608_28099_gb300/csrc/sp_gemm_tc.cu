@@ -1063,11 +1063,20 @@ TcPlan tc_plan(int M, int N, int K, int n_sm, size_t y_capacity_bytes, bool lo, 
     }
     // The pair kernel takes 128-row tiles with the lo plane and 256-row tiles
     // (measured at d = 4096, 1024 rows: Q/K/V 79.9 -> 63.2 us, gate/up 159.4 ->
-    // 124.9 us).  128-row plain tiles are bound by the weights: there the cluster's
-    // start costs as much as the smaller activation half gives until an item has
-    // about 64 k-blocks (4B down at 22: 11.4 -> 11.9 us, 27B down at 91: 32.0 -> 30.8).
-    p.pair = p.n_tiles % 2 == 0 && n_sm >= 2 &&
-             (p.bn == 256 || (p.bn == 128 && (lo || p.kb_per_split >= 64)));
+    // 124.9 us) where there is work behind the cluster's start, which costs 1-1.5 us
+    // of a kernel: more items than pairs of CTAs, whose epilogues then overlap, or
+    // enough k-blocks in an item.  Whole calls without that rule -> with it: d = 1024
+    // (2 to 6 k-blocks an item) 80 rows 61.6 -> 59.5 us, 128 rows 64.6 -> 60.6, 256 rows
+    // 79.5 -> 75.6; d = 2048 (4 to 11) 128 rows 72.8 -> 70.9; d = 4096 (16 and 22) 128 rows
+    // 127.5 -> 126.6.  The line at 20 k-blocks: items of 22 gain 0.7-1.0 us on pairs, of 16
+    // lose 0.6-1.4; 256-row tiles: of 6 lose 1.9 or gain 0.5, of 11 gain 0.9.  128-row plain
+    // tiles are bound by the weights and gain later: a call with items of 64 loses up to
+    // 1.4 %, of 72 gains 0.5 %, of 91 1.7 %, of 128 2.6 %.
+    const int pair_items = p.m_tiles * (p.n_tiles / 2) * p.splits;
+    const bool rows_of_pairs = p.bn == 256 || (p.bn == 128 && lo);
+    p.pair = p.n_tiles % 2 == 0 && n_sm >= 2 && p.bn >= 128 &&
+             ((rows_of_pairs && pair_items > n_sm / 2) ||
+              p.kb_per_split >= (p.bn == 256 ? 8 : lo ? 20 : 72));
     if (sched == 1) return p;
     if (sched == 2 || (waves > 1 && fill < 0.8)) {
         const long long U = (long long)tiles * p.n_kb;
