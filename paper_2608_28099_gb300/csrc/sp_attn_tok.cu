@@ -27,13 +27,14 @@
 // more to rounding than the queries-on-M kernel's one per 64.  Against that, the row
 // sums (fp32) are over the probabilities as rounded: an error e of a token's weight
 // then moves the output by e (v - o) instead of e v, never more on average over values of
-// one distribution (sum w^2 - 2 sum w^3 + (sum w^2)^2 <= sum w^2); and sequences of up to
-// 512 tokens have the lo plane (256 from 33 rows on, where holding the K slot costs
-// 2-3 % of a call beyond).  Relative error of the output, 4 rows of 32 heads: 100 tokens
-// 1.45e-3 (queries on M), 1.53e-3 (this kernel with neither), 1.00e-3 (now); 300 tokens
-// 1.64e-3, 1.66e-3, 1.41e-3; 1000 tokens 1.66e-3, 1.67e-3, 1.63e-3; 4000 tokens 1.64e-3 in
-// all.  The sums cost nothing that can be measured, the lo plane 0.3-0.6 % of a call of
-// up to 32 rows that has one and about 0.2 % of others.
+// one distribution (sum w^2 - 2 sum w^3 + (sum w^2)^2 <= sum w^2); and sequences of two to
+// eight tiles, up to 512 tokens, have the lo plane (two to four from 33 rows on, where
+// holding the K slot costs 2-3 % of a call beyond).  Relative error of the output, 4 rows
+// of 32 heads: 100 tokens 1.45e-3 (queries on M), 1.53e-3 (this kernel with neither),
+// 1.00e-3 (now); 300 tokens 1.64e-3, 1.66e-3, 1.41e-3; 1000 tokens 1.66e-3, 1.67e-3,
+// 1.63e-3; 4000 tokens 1.64e-3 in all.  The sums cost nothing that can be measured, the
+// lo plane 0 to 4 % of the attention of a batch that has it (124 sequences of 92 to 155
+// tokens, paged, 4 / 16 / 32 rows: 37.2 / 39.0 / 51.5 -> 38.7 / 39.2 / 51.4 us).
 // An MMA costs the padded row count instead of 128 columns (40 cycles at 32 rows,
 // shared-memory bandwidth of the token operand), and a step of 128 tokens takes
 // 1.2-1.4 us while all SMs stream: HBM-bound (7 TB/s between a segment's first and
@@ -257,7 +258,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr uint32_t TMEM_COLS = NR <= 32 ? 128 : 256;
     static_assert(NR % 16 == 0 && NR <= 64, "query rows");
     constexpr bool LO_IN_LINE = NR <= 32;        // P's lo plane in P's lines, else in the K slot
-    constexpr int LO_TILES = LO_IN_LINE ? 8 : 4; // sequences (tiles) that have one: 512 or 256 tokens
+    constexpr int LO_TILES = LO_IN_LINE ? 8 : 4; // tiles of the longest sequence that has one
+    // (a sequence of one tile needs none: one maximum in either kernel)
+    auto has_lo = [](const Seg &sg) { return sg.nt >= 2 && sg.nt <= LO_TILES; };
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     TokBars *bars = (TokBars *)(smem + OFF_BAR);
@@ -534,7 +537,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     mma_bf16(d, ak, bq, idesc_s, kk > 0 ? 1u : 0u);
                     if (q_lo) mma_bf16(d, ak, bq + (uint64_t)(NR * 256 >> 4), idesc_s, 1u);
                 }
-                if (LO_IN_LINE || ws.i > 0 || ws.sg.nt > LO_TILES) mma_commit(&bars->k_empty[rk.slot]);
+                if (LO_IN_LINE || ws.i > 0 || !has_lo(ws.sg)) mma_commit(&bars->k_empty[rk.slot]);
                 mma_commit(&bars->s_full[sbuf]);
                 if (ws.i == ws.n - 1) mma_commit(&bars->q_empty[rq.slot]);
             }
@@ -561,7 +564,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (kk < TT / 16 || two)
                         mma_bf16(tmem + O_COL, dv + (uint64_t)(kk * (2 * GROUP_STRIDE >> 4)),
                                  dp0 + (uint64_t)(kk * (2048 >> 4)), idesc_o, (w.i > 0 || kk > 0) ? 1u : 0u);
-                if (w.i == 0 && w.sg.nt <= LO_TILES) {
+                if (w.i == 0 && has_lo(w.sg)) {
                     const uint64_t dl = LO_IN_LINE ? dp0 + (64 >> 4) : dl0 + (uint32_t)(rp.slot * (SLOT >> 4));
 #pragma unroll
                     for (int kk = 0; kk < STEP / 16; ++kk)
@@ -700,12 +703,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (n > 0 && !pv_waited)
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->pv_done, (uint32_t)(n - 1) & 1, abort));
                 uint8_t *prow = smem + lay.off_p + (tok >> 3) * 1024 + (tok & 7) * 128;
+                const bool with_lo = i == 0 && has_lo(sg);  // uniform
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     float(&s)[W] = sv[c];
 #pragma unroll
                     for (int j8 = 0; j8 < W; j8 += 8) {
-                        uint32_t pk[4];
+                        uint32_t pk[4], lo[4];
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int j = j8 + 4 * h, cj = c * W + j;
@@ -724,14 +728,28 @@ __global__ void __launch_bounds__(THREADS, 1)
                                  __uint_as_float(u1 & 0xffff0000u));
                             pk[2 * h] = u0;
                             pk[2 * h + 1] = u1;
+                            if (LO_IN_LINE && with_lo) {
+                                const float e0 = p0 - __uint_as_float(u0 << 16);
+                                const float e1 = p1 - __uint_as_float(u0 & 0xffff0000u);
+                                const float e2 = p2 - __uint_as_float(u1 << 16);
+                                const float e3 = p3 - __uint_as_float(u1 & 0xffff0000u);
+                                add2(l[cj], l[cj + 1], l[cj], l[cj + 1], e0, e1);
+                                add2(l[cj + 2], l[cj + 3], l[cj + 2], l[cj + 3], e2, e3);
+                                lo[2 * h] = pack_bf16(e0, e1);
+                                lo[2 * h + 1] = pack_bf16(e2, e3);
+                            }
                         }
                         const int c16 = (cb + c * W + j8) >> 3;  // 16-byte chunk of the line
                         st_shared_v4(prow + ((c16 ^ (tok & 7)) << 4), pk[0], pk[1], pk[2], pk[3]);
+                        if (LO_IN_LINE && with_lo)
+                            st_shared_v4(prow + (((c16 + 4) ^ (tok & 7)) << 4), lo[0], lo[1], lo[2], lo[3]);
                     }
                 }
-                if (i == 0 && sg.nt <= LO_TILES) {  // uniform
-                    // (every step takes the next of the nk K slots)
-                    uint8_t *lrow = LO_IN_LINE ? prow : prow + (lay.off_k - lay.off_p) + n % lay.nk * SLOT;
+                if (!LO_IN_LINE && with_lo) {
+                    // the lo plane in a pass of its own, in which the exponentials are formed
+                    // again (in the one above its values do not fit the registers: 140 bytes
+                    // of spills at 64 rows); every step takes the next of the nk K slots
+                    uint8_t *lrow = prow + (lay.off_k - lay.off_p) + n % lay.nk * SLOT;
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
 #pragma unroll
@@ -744,7 +762,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 e[j] = p - __bfloat162float(__float2bfloat16_rn(p));
                                 l[c * W + j8 + j] += e[j];
                             }
-                            const int c16 = ((cb + c * W + j8) >> 3) + (LO_IN_LINE ? 4 : 0);
+                            const int c16 = (cb + c * W + j8) >> 3;
                             st_shared_v4(lrow + ((c16 ^ (tok & 7)) << 4), pack_bf16(e[0], e[1]), pack_bf16(e[2], e[3]),
                                          pack_bf16(e[4], e[5]), pack_bf16(e[6], e[7]));
                         }
