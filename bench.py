@@ -55,7 +55,8 @@ FLUSH_BYTES = 256 << 20
 # The attention kernel's figure includes the output projection's weights that its
 # CTAs prefetch into L2 as they finish (52.4 MB on 27b_long, 21 MB on 4b): the next kernel's
 # bytes, issued early.
-TRAFFIC_BYTES = {("27b_long", "attention"): 1132972800, ("4b", "attention"): 99060992}
+TRAFFIC_BYTES = {("27b_long", "attention"): 1132929408, ("4b", "attention"): 98901504,
+                 ("8b_paged", "attention"): 1217012224}
 
 
 def parse_args():
