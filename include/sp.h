@@ -265,16 +265,17 @@ enum {
                                  always, 4 = plain bf16 except Q/K/V            */
     SP_OPT_DEBUG_STALL = 8,   /* test of the failure path: 1 = in the next
                                  sp_classify only, the first CTA of the output
-                                 projection (unless it runs on the persistent
-                                 stream-K schedule) never loads its first k-block, so its
-                                 tensor-core wait runs out; that launch's waits
+                                 projection (on one-CTA tiles or pairs of CTAs,
+                                 not on stream-K) never loads its first k-block,
+                                 so its tensor-core wait runs out; that launch's waits
                                  give up after 1 ms, the kernel drains its copies,
                                  frees TMEM and returns, and sp_check_status
                                  reports SP_DEV_TIMEOUT (that call's logits are
                                  invalid, the handle stays usable).  Resets
                                  itself after that call                          */
-    SP_OPT_GEMM_SCHEDULE = 9, /* tensor-core projections: 0 = automatic, 1 = one
-                                 CTA per (weight tile, K split), 2 = persistent
+    SP_OPT_GEMM_SCHEDULE = 9, /* tensor-core projections: 0 = automatic, 1 = whole
+                                 (weight tile, K split) items, by one CTA each
+                                 or by pairs of CTAs in turn, 2 = persistent
                                  stream-K (one CTA per SM, an even share of the
                                  (tile, k-block) units each) wherever its partial
                                  planes fit the handle's scratch.  Changes the

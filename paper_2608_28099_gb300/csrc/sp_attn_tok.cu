@@ -37,8 +37,8 @@
 // tokens, paged, 4 / 16 / 32 rows: 37.2 / 39.0 / 51.5 -> 38.7 / 39.2 / 51.4 us).
 // An MMA costs the padded row count instead of 128 columns (40 cycles at 32 rows,
 // shared-memory bandwidth of the token operand), and a step of 128 tokens takes
-// 1.2-1.4 us while all SMs stream: HBM-bound (7 TB/s between a segment's first and
-// last step) instead of bound by the 1.5 us chain per 64 tokens of the
+// 1.2-1.4 us while all SMs stream (1.2 GB at 6.0 TB/s, 0.89 of the copy rate, in the 8B
+// paged call's kernel: HBM-bound) instead of the 1.5 us chain per 64 tokens of the
 // queries-on-M kernel.  S^T is double-buffered in TMEM: the scores of step n + 1
 // are ready when the softmax of step n ends.  The queries of the next segment are
 // loaded by warps of their own into the other query buffer, so the pipeline does

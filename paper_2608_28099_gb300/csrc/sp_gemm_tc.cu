@@ -21,8 +21,9 @@
 //    TMEM, all eight warps the epilogue (warp w: TMEM lanes 32 (w & 3).., the
 //    column chunks of half w >> 2).  A gate/up projection with one K split can
 //    apply SwiGLU in the epilogue instead of writing partials.
-//  * pair kernel, in the tile kernel's place for the larger tiles: two CTAs per
-//    MMA (cta_group::2), the same (tile, K split) items, persistent.
+//  * pair kernel, in the tile kernel's place for the larger tiles where there is work
+//    behind its start (tc_plan): two CTAs per MMA (cta_group::2), the same (tile, K
+//    split) items, persistent.
 //  * persistent stream-K kernel, for tile counts that fill the SMs badly:
 //    one CTA per SM owns the contiguous (tile, k-block) units [c L, (c+1) L)
 //    in tile-major order.  Its weight and activation rings run across tile
@@ -72,8 +73,9 @@ struct TcArgs {
     float *y;         // [split][M][N]
     size_t split_stride;
     int *status;
-    // failure-path test: CTA (0, 0, 0) never loads its first k-block, so its
-    // MMA warp's wait runs out; every wait of the launch gives up after wait_ns
+    // failure-path test: CTA (0, 0, 0), or rank 0 of the first pair, never loads its
+    // first k-block, so its MMA warp's wait runs out; every wait of the launch gives up
+    // after wait_ns
     int inject_stall;
     unsigned long long wait_ns;
     // SwiGLU epilogue (glu_f > 0, one K split): weight tile t holds gate rows
@@ -390,7 +392,8 @@ cudaError_t launch_tile(const CUtensorMap &mw, const CUtensorMap &mh, const CUte
 // writes and reads a third less shared memory per MMA.  Persistent: each pair
 // takes items (row tile, weight tile pair, K split) in turn, with two
 // accumulators in TMEM, so the epilogue of one overlaps the MMAs of the next.
-// Bound by the tensor pipe (the one-CTA tile kernel by shared-memory bandwidth
+// Bound by the tensor pipe (busy for 64-70 % of a cold launch of 1024 rows, whose items
+// do not divide the pairs; the one-CTA tile kernel by shared-memory bandwidth
 // and its exposed epilogue): 4096 rows at d = 4096, Q/K/V hi + lo 325 -> 240 us
 // (1.7 PFLOP/s issued), gate/up 538 -> 440 us (1.88 PFLOP/s), down 303 -> 250 us.
 constexpr int PAIR_THREADS = 384;  // warps 0-7 epilogue, 8 TMA, 9 MMA (rank 0), 10 TMEM
