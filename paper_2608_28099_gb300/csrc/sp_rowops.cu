@@ -374,7 +374,8 @@ __global__ void swiglu_kernel(PartIn y, int M, int f, int blk, ActOut a) {
 // Latency-bound: a block is one dependent round trip for its rows, one for the
 // count and one for the sum (3-4 us in all), so the blocks should be few and
 // large: one row group (1024 columns a block, rows four at a time) where that
-// covers the SMs, more groups only where it does not.  With four groups
+// covers the SMs, more groups only where it does not (a group sums its rows and
+// takes its classes, so it is of use with several of either).  With four groups
 // everywhere 96 states of one row took 17.4 us (5 waves of blocks whose threads
 // mostly had no row), 128 of four rows 23.2, 64 of 16 rows 15.1 and 256 of 16
 // rows 48.8 (d = 4096); now 5.8, 8.7, 9.9 and 31.2 us (the last reads 134 MB).
@@ -760,10 +761,17 @@ cudaError_t launch_readout(PartIn y, const float *h1, const float *head_w, const
     if (!sr) sr = d;
     if (n_tasks < 1) n_tasks = 1;
     // row groups: none while the grid covers the SMs (see the kernel), else up
-    // to one per row
+    // to one per row or, since a group also takes its own classes, up to one per
+    // kReadoutHeads classes.  Counted by rows alone, a pooled row with many classes
+    // ran them four at a time in a quarter of the blocks: whole calls at d = 1024,
+    // last row, 1 x 100 classes 50.4 us -> 40.4, 1 x 1000 213.5 -> 102.1, 32 x 300
+    // 97.2 -> 67.5; with up to 4 classes nothing changes.  Groups on a grid that
+    // covers the SMs gain only past ~100 classes and lose before (d = 4096,
+    // 256 x 33: 113 -> 124 us), so that line stays.
     const int rows = pool == SP_POOL_LAST ? 1 : k;
+    const int most = max(rows, ceil_div(C, kReadoutHeads));
     int RG = 1;
-    while (RG < 4 && RG < rows && ceil_div(d, 4 * kReadoutThreads / RG) * B < sm_count_cached()) RG *= 2;
+    while (RG < 4 && RG < most && ceil_div(d, 4 * kReadoutThreads / RG) * B < sm_count_cached()) RG *= 2;
     const int chunks = ceil_div(d, 4 * kReadoutThreads / RG);
     float *ss = g_final ? scratch + (size_t)B * chunks * C : nullptr;
 #define SP_READOUT_P(RR, PP)                                                                        \

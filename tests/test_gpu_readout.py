@@ -14,6 +14,10 @@ pytestmark = pytest.mark.gpu
     (1, 2, 1032, 5, wl.POOL_MEAN, True),      # two groups, eight columns in the last chunk
     (3, 7, 520, 21, wl.POOL_MEAN, False),     # four groups, more classes than one pass
     (2, 32, 256, 17, wl.POOL_LAST, True),     # one pooled row of many, classes past 4 x 4
+    (2, 4, 264, 4, wl.POOL_LAST, False),      # one pooled row, one pass of classes: one group
+    (2, 4, 1032, 5, wl.POOL_LAST, False),     # one pooled row, two groups by its classes
+    (1, 1, 520, 9, wl.POOL_MEAN, True),       # one row, four groups by its classes
+    (3, 1, 1032, 300, wl.POOL_MEAN, False),   # the same, many passes
     (160, 5, 128, 3, wl.POOL_MEAN, True),     # one group, rows past four
     (160, 16, 128, 33, wl.POOL_MEAN, False),  # one group, classes past a warp
 ])
@@ -29,3 +33,27 @@ def test_readout_block_shapes(B, k, d, C, pool, lm_head):
     compare(gpu, ref, label="readout")
     assert np.array_equal(gpu, run.logits())  # counters are clear again, the sum order is fixed
     run.close()
+
+
+@pytest.mark.parametrize("k,C,pool,groups", [
+    (4, 4, wl.POOL_LAST, 1), (4, 5, wl.POOL_LAST, 2), (4, 9, wl.POOL_LAST, 4), (1, 300, wl.POOL_MEAN, 4),
+    (4, 2, wl.POOL_MEAN, 4), (2, 2, wl.POOL_MEAN, 2),
+])
+def test_row_groups_follow_rows_and_classes(k, C, pool, groups):
+    """A small batch: as many groups as the pooled rows or the classes can use."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    w = wl.custom(wl.Shape(256, 4, 2, 32, 64, k, C, pool=pool), np.array([5, 9]), wl.LAYOUT_PAGED, 77,
+                  rows_per_seq=True)
+    run = GpuRun(w)
+    for _ in range(3):  # (a process's first trace can be empty)
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            run.logits()
+            torch.cuda.synchronize()
+        names = " ".join(e.name for e in prof.events())
+        if "readout_kernel" in names:
+            break
+    else:
+        pytest.skip("no CUDA trace in this process (another profiler holds it)")
+    run.close()
+    assert f"readout_kernel<{groups}," in names, names
